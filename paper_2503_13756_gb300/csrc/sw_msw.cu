@@ -5,16 +5,21 @@
 // pair is formed: O(n^2 M) per pair.
 //
 // Design (GB300): the per-angle terms are squared differences summed
-// directly in FP32 (no Gram-matrix cancellation).  One CTA takes one pair
-// and a block of R rows k of the query against all n columns k' of the
-// template, staging the query rows [R][PC] and the template columns
-// transposed [PC][n+1] in shared memory, PC levels at a time; each thread
-// owns the columns k' = t, t + 256, ... and R accumulators per column.  The
-// block's terms then go to shared memory, each thread takes rotations
-// l = t, t + 256, ... and the maximum over its rows of E[k][(k - l) mod n],
-// and the blocks of a pair meet in an atomic max on the pair's curve (the
-// terms are >= 0, so their float bits order as integers; the maximum does
-// not depend on the order).  A second kernel takes the argmin per pair.
+// directly in FP32 (no Gram-matrix cancellation), level by level.  One CTA
+// takes one pair and a tile of 64 rows k of the query against 64 CC <= 256
+// columns k' of the template (all of them up to n = 256), staged 32 levels at
+// a time; a warp owns eight of the rows and each lane 2 CC columns, as CC
+// adjacent pairs, so that the difference and the square of two columns are
+// one two-wide FP32 operation each.  The query values are staged twice side
+// by side (the two-wide operand without a move) and the template's negated,
+// columns transposed.  The tile's terms then go to shared memory, each thread
+// takes rotations l = t, t + 256, ... and the maximum over the tile's rows of
+// E[k][(k - l) mod n], and the tiles of a pair meet in an atomic max on the
+// pair's curve (the terms are >= 0, so their float bits order as integers;
+// the maximum does not depend on the order).  A second kernel takes the
+// argmin per pair.
+//
+// Bound: two FP32 operations per level and column pair (k, k').
 #include "sw_internal.cuh"
 #include "swalign.h"
 
@@ -22,28 +27,43 @@ namespace swk {
 namespace {
 
 constexpr int kMswThreads = 256;
-constexpr int kMswPC = 32;  // levels per stage (a multiple of 4)
+constexpr int kMswPC = 32;     // levels per stage (even)
+constexpr int kMswWR = 8;      // rows per warp
+constexpr int kMswR = kMswWR * kMswThreads / 32;  // rows per CTA
 
-template <int R, int NC>
-__global__ void __launch_bounds__(kMswThreads)
+constexpr int kMswUS = kMswR + 2;  // staged row stride (16-byte rows, few bank conflicts)
+
+// Shared memory: the staged tiles Us [PC][R + 2] of (u, u) and Vt [PC][64 CC + 2]
+// of -v, then, in the same place, the terms Eb [R][64 CC]; and the template
+// columns' offsets [64 CC].
+size_t msw_smem(int CC)
+{
+    const size_t stage = 8 * (size_t)kMswPC * kMswUS + 4 * (size_t)kMswPC * (64 * CC + 2);
+    const size_t terms = 4 * (size_t)kMswR * 64 * CC;
+    return (stage > terms ? stage : terms) + 4 * (size_t)64 * CC;
+}
+
+template <int CC>
+__global__ void __launch_bounds__(kMswThreads, 2)
 k_msw(MswArgs A)
 {
-    extern __shared__ float sms[];
+    constexpr int W = 64 * CC, R = kMswR, VS = W + 2;
+    extern __shared__ __align__(16) float sms[];
     const int n = A.n, M = A.M;
-    const int np1 = n + 1;
-    float *Us = sms;                   // [R][kMswPC]
-    float *Vt = Us + R * kMswPC;       // [kMswPC][n + 1]
-    float *Eb = Vt + kMswPC * np1;     // [R][n]
-    float *offt = Eb + R * n;          // [n] template column offsets
+    float2 *Us = reinterpret_cast<float2 *>(sms);  // [kMswPC][kMswUS]
+    float *Vt = sms + 2 * kMswPC * kMswUS;              // [kMswPC][VS]
+    float *Eb = sms;                               // [R][W]
+    constexpr int kStage = 2 * kMswPC * kMswUS + kMswPC * VS, kTerms = R * W;
+    float *offt = sms + (kStage > kTerms ? kStage : kTerms);  // [W]
     __shared__ float offq[R];
     const int pair = blockIdx.x;
     const int i = pair / A.Nt, j = pair % A.Nt;
-    const int k0 = blockIdx.y * R;
-    const int t = threadIdx.x;
+    const int k0 = blockIdx.y * R, c0 = blockIdx.z * W;
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const float *Qi = A.q + (size_t)i * n * M;
     const float *Qj = A.t + (size_t)j * n * M;
-    // centring offsets <a, e_k> (translation): query rows here, template
-    // columns folded into the staging below
+    // centring offsets <a, e_k> (translation): subtracted in the staging
+    // below (FP64 is scarce: once per column, not once per staged level)
     const double2 *cs = A.cs64;
     const double aix = A.translation ? A.ctr_q[2 * i] : 0.0;
     const double aiy = A.translation ? A.ctr_q[2 * i + 1] : 0.0;
@@ -53,75 +73,97 @@ k_msw(MswArgs A)
         const int k = k0 + t;
         offq[t] = k < n ? (float)(aix * cs[k].x + aiy * cs[k].y) : 0.f;
     }
-    // once per column (FP64 is scarce: not once per staged level)
-    for (int kk = t; kk < n; kk += kMswThreads)
-        offt[kk] = A.translation ? (float)(ajx * cs[kk].x + ajy * cs[kk].y) : 0.f;
-    float acc[NC][R];
+    for (int c = t; c < W; c += kMswThreads) {
+        const int kk = c0 + c;
+        offt[c] = A.translation && kk < n ? (float)(ajx * cs[kk].x + ajy * cs[kk].y) : 0.f;
+    }
+    float2 acc[kMswWR][CC];
 #pragma unroll
-    for (int c = 0; c < NC; ++c)
+    for (int r = 0; r < kMswWR; ++r)
 #pragma unroll
-        for (int r = 0; r < R; ++r) acc[c][r] = 0.f;
+        for (int c = 0; c < CC; ++c) acc[r][c] = make_float2(0.f, 0.f);
     __syncthreads();
+    const bool vec = (M & 3) == 0;  // every row starts on 16 bytes
     for (int p0 = 0; p0 < M; p0 += kMswPC) {
         const int pc = min(kMswPC, M - p0);
-        // query rows: Us[r][p] (zero outside), centred
-        for (int e = t; e < R * kMswPC; e += kMswThreads) {
-            const int r = e / kMswPC, p = e % kMswPC, k = k0 + r;
-            Us[e] = (k < n && p < pc) ? Qi[(size_t)k * M + p0 + p] - offq[r] : 0.f;
-        }
-        // template columns transposed: Vt[p][k'] (zero outside), centred
-        for (int e = t; e < n * kMswPC; e += kMswThreads) {
-            const int kk = e / kMswPC, p = e % kMswPC;
-            float v = 0.f;
-            if (p < pc) v = Qj[(size_t)kk * M + p0 + p] - offt[kk];
-            Vt[p * np1 + kk] = v;
+        // (u, u) and -v, centred, zero outside (zeros add nothing); four
+        // levels per load where the rows keep 16-byte alignment
+        constexpr int P4 = kMswPC / 4;
+        for (int e = t; e < (R + W) * P4; e += kMswThreads) {
+            const int row = e / P4, p = 4 * (e % P4);
+            const bool is_q = row < R;
+            const int c = is_q ? row : row - R;
+            const int kk = (is_q ? k0 : c0) + c;
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (kk < n && p < pc) {
+                const float *src = (is_q ? Qi : Qj) + (size_t)kk * M + p0 + p;
+                const float o = is_q ? offq[c] : offt[c];
+                if (vec) {
+                    x = __ldg(reinterpret_cast<const float4 *>(src));
+                    x = make_float4(x.x - o, x.y - o, x.z - o, x.w - o);
+                } else {
+                    x.x = src[0] - o;
+                    if (p + 1 < pc) x.y = src[1] - o;
+                    if (p + 2 < pc) x.z = src[2] - o;
+                    if (p + 3 < pc) x.w = src[3] - o;
+                }
+            }
+            if (is_q) {
+                Us[p * kMswUS + c] = make_float2(x.x, x.x);
+                Us[(p + 1) * kMswUS + c] = make_float2(x.y, x.y);
+                Us[(p + 2) * kMswUS + c] = make_float2(x.z, x.z);
+                Us[(p + 3) * kMswUS + c] = make_float2(x.w, x.w);
+            } else {
+                Vt[p * VS + c] = -x.x;
+                Vt[(p + 1) * VS + c] = -x.y;
+                Vt[(p + 2) * VS + c] = -x.z;
+                Vt[(p + 3) * VS + c] = -x.w;
+            }
         }
         __syncthreads();
-        // four levels at a time: one 16-byte read of each query row (the
-        // staged tiles are zero past pc, and zeros add nothing)
-        for (int p = 0; p < pc; p += 4) {
-            float v[NC][4];
+#pragma unroll 2
+        for (int p = 0; p < pc; ++p) {
+            float2 v[CC];
 #pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                const int kk = t + c * kMswThreads;
+            for (int c = 0; c < CC; ++c)
+                v[c] = *reinterpret_cast<const float2 *>(Vt + p * VS + 64 * c + 2 * lane);
+            const float4 *up = reinterpret_cast<const float4 *>(Us + p * kMswUS + kMswWR * warp);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) v[c][q] = kk < n ? Vt[(p + q) * np1 + kk] : 0.f;
-            }
+            for (int r2 = 0; r2 < kMswWR / 2; ++r2) {
+                const float4 uu = up[r2];  // two rows
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const float4 u = *reinterpret_cast<const float4 *>(Us + r * kMswPC + p);
-#pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    float d = u.x - v[c][0];
-                    acc[c][r] = fmaf(d, d, acc[c][r]);
-                    d = u.y - v[c][1];
-                    acc[c][r] = fmaf(d, d, acc[c][r]);
-                    d = u.z - v[c][2];
-                    acc[c][r] = fmaf(d, d, acc[c][r]);
-                    d = u.w - v[c][3];
-                    acc[c][r] = fmaf(d, d, acc[c][r]);
+                for (int c = 0; c < CC; ++c) {
+                    const float2 d0 = __fadd2_rn(make_float2(uu.x, uu.y), v[c]);
+                    acc[2 * r2][c] = __ffma2_rn(d0, d0, acc[2 * r2][c]);
+                    const float2 d1 = __fadd2_rn(make_float2(uu.z, uu.w), v[c]);
+                    acc[2 * r2 + 1][c] = __ffma2_rn(d1, d1, acc[2 * r2 + 1][c]);
                 }
             }
         }
         __syncthreads();
     }
-    // ---- block terms to shared memory, then diagonal maxima per rotation
+    // ---- tile terms to shared memory, then diagonal maxima per rotation
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {
-        const int kk = t + c * kMswThreads;
-        if (kk < n)
+    for (int r = 0; r < kMswWR; ++r)
 #pragma unroll
-            for (int r = 0; r < R; ++r) Eb[r * n + kk] = acc[c][r];
-    }
+        for (int c = 0; c < CC; ++c)
+            *reinterpret_cast<float2 *>(Eb + (kMswWR * warp + r) * W + 64 * c + 2 * lane) =
+                acc[r][c];
     __syncthreads();
-    const int rows = min(R, n - k0);
+    const int rows = min(R, n - k0), cols = min(W, n - c0);
     unsigned *curve = reinterpret_cast<unsigned *>(A.curve) + (size_t)pair * n;
     for (int l = t; l < n; l += kMswThreads) {
         float mx = 0.f;
-        for (int r = 0; r < rows; ++r) {
-            int kk = k0 + r - l;
-            kk += kk < 0 ? n : 0;
-            mx = fmaxf(mx, Eb[r * n + kk]);
+        // row r takes the template column (k0 + r - l) mod n: the tile's
+        // rows where it lies in the tile form at most two runs
+        int cb = k0 - l - c0;
+        cb += k0 < l ? n : 0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h, cb -= n) {
+            const int r0 = max(0, -cb), r1 = min(rows, cols - cb);
+            const float *Er = Eb + cb;
+#pragma unroll 4
+            for (int r = r0; r < r1; ++r) mx = fmaxf(mx, Er[r * (W + 1)]);
         }
         atomicMax(curve + l, __float_as_uint(mx));
     }
@@ -192,14 +234,15 @@ __global__ void k_msw_decide(MswArgs A)
     }
 }
 
-template <int R, int NC>
-cudaError_t launch_rows(const MswArgs &a, cudaStream_t st)
+template <int CC>
+cudaError_t launch_tiles(const MswArgs &a, int nblk, cudaStream_t st)
 {
-    const size_t smem = sizeof(float) * ((size_t)R * kMswPC + (size_t)kMswPC * (a.n + 1) +
-                                         (size_t)R * a.n + a.n);
-    cudaFuncSetAttribute(k_msw<R, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    dim3 grid(a.Nq * a.Nt, (a.n + R - 1) / R);
-    k_msw<R, NC><<<grid, kMswThreads, smem, st>>>(a);
+    const size_t smem = msw_smem(CC);
+    cudaError_t e = cudaFuncSetAttribute(k_msw<CC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e != cudaSuccess) return e;
+    const dim3 grid(a.Nq * a.Nt, (a.n + kMswR - 1) / kMswR, nblk);
+    k_msw<CC><<<grid, kMswThreads, smem, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -213,9 +256,14 @@ cudaError_t launch_msw(const MswArgs &args, cudaStream_t st)
     a.dalpha = 6.283185307179586 / a.n;
     cudaError_t e = cudaMemsetAsync(a.curve, 0, sizeof(float) * (size_t)a.Nq * a.Nt * a.n, st);
     if (e != cudaSuccess) return e;
-    if (a.n <= 256) e = launch_rows<64, 1>(a, st);
-    else if (a.n <= 512) e = launch_rows<32, 2>(a, st);
-    else e = launch_rows<16, 4>(a, st);
+    // the columns in equal blocks of at most 256
+    const int nblk = (a.n + 255) / 256;
+    switch ((a.n + 64 * nblk - 1) / (64 * nblk)) {
+    case 1: e = launch_tiles<1>(a, nblk, st); break;
+    case 2: e = launch_tiles<2>(a, nblk, st); break;
+    case 3: e = launch_tiles<3>(a, nblk, st); break;
+    default: e = launch_tiles<4>(a, nblk, st); break;
+    }
     if (e != cudaSuccess) return e;
     const int threads = 256;
     const long long warps = (long long)a.Nq * a.Nt;
