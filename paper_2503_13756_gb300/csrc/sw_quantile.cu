@@ -18,12 +18,16 @@
 // counts the levels below its right node and the bins whose count grows put
 // their index at their first level; a warp maximum scan over the levels then
 // gives every level its bin, without divergence.  No FP64 on this path.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "sw_internal.cuh"
 
 namespace swk {
 namespace {
+
+namespace cg = cooperative_groups;
 
 constexpr int kQThreads = 256;  // 8 warps
 
@@ -454,27 +458,38 @@ k_quantiles(const float *__restrict__ proj, int n, int B, int M, float h, int le
     }
 }
 
-// Centring vector and centred norm (public sw_quantiles outputs).  One block
-// per image; FP64 accumulation.
-__global__ void k_center_norm(const float *__restrict__ q, int n, int M,
-                              const double2 *__restrict__ cs64, double *__restrict__ center,
-                              double *__restrict__ norm)
+// Centring vector and centred norm (public sw_quantiles outputs), FP64
+// accumulation.  A cluster of CTAs per image shares its rows; the partial
+// sums meet in the shared memory of the cluster's CTAs, added in rank order
+// by every CTA.  Bound by FP64 issue, so a row costs only the additions of
+// its quantiles and two fused multiply-adds (no division or warp reduction
+// per row: those were four fifths of the instructions), the norm is skipped
+// when it is not wanted, and every SM has rows (64 images on one CTA each
+// left 88 of 152 SMs idle).
+__global__ void __launch_bounds__(256)
+k_center_norm(const float *__restrict__ q, int n, int M, const double2 *__restrict__ cs64,
+              double *__restrict__ center, double *__restrict__ norm)
 {
     __shared__ double red[3][32];
-    __shared__ double s_a[2];
-    const int imgi = blockIdx.x;
+    __shared__ double part[3];  // this CTA's sums: a (x, y), norm
+    cg::cluster_group cl = cg::this_cluster();
+    const int S = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const int imgi = blockIdx.x / S;
     const float *qi = q + (size_t)imgi * n * M;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    // a = (2/n) sum_k ubar_k (cos, sin),  ubar_k = mean_p q[k][p]
+    // a = (2/n) sum_k ubar_k (cos, sin),  ubar_k = mean_p q[k][p]: every lane
+    // weights its own share of each row's sum
     double ax = 0.0, ay = 0.0;
-    for (int k = warp; k < n; k += nw) {
+    for (int k = rank * nw + warp; k < n; k += S * nw) {
         double s = 0.0;
         for (int p = lane; p < M; p += 32) s += (double)qi[(size_t)k * M + p];
+        ax += s * cs64[k].x;
+        ay += s * cs64[k].y;
+    }
 #pragma unroll
-        for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-        const double ub = s / M;
-        ax += ub * cs64[k].x;
-        ay += ub * cs64[k].y;
+    for (int off = 16; off; off >>= 1) {
+        ax += __shfl_xor_sync(0xffffffffu, ax, off);
+        ay += __shfl_xor_sync(0xffffffffu, ay, off);
     }
     if (lane == 0) {
         red[0][warp] = ax;
@@ -487,32 +502,50 @@ __global__ void k_center_norm(const float *__restrict__ q, int n, int M,
             sx += red[0][w];
             sy += red[1][w];
         }
-        s_a[0] = sx * 2.0 / n;
-        s_a[1] = sy * 2.0 / n;
+        part[0] = sx;
+        part[1] = sy;
     }
-    __syncthreads();
-    const double a0 = s_a[0], a1 = s_a[1];
-    double acc = 0.0;
-    for (int k = warp; k < n; k += nw) {
-        const double off = a0 * cs64[k].x + a1 * cs64[k].y;
-        for (int p = lane; p < M; p += 32) {
-            const double d = (double)qi[(size_t)k * M + p] - off;
-            acc += d * d;
+    cl.sync();
+    double a0 = 0.0, a1 = 0.0;
+    for (int r = 0; r < S; ++r) {
+        const double *o = cl.map_shared_rank(part, r);
+        a0 += o[0];
+        a1 += o[1];
+    }
+    a0 = a0 * 2.0 / ((double)n * M);
+    a1 = a1 * 2.0 / ((double)n * M);
+    if (norm) {
+        double acc = 0.0;
+        for (int k = rank * nw + warp; k < n; k += S * nw) {
+            const double off = a0 * cs64[k].x + a1 * cs64[k].y;
+            for (int p = lane; p < M; p += 32) {
+                const double d = (double)qi[(size_t)k * M + p] - off;
+                acc += d * d;
+            }
         }
-    }
 #pragma unroll
-    for (int off = 16; off; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if (lane == 0) red[2][warp] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < nw; ++w) s += red[2][w];
+        for (int off = 16; off; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+        if (lane == 0) red[2][warp] = acc;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double s = 0.0;
+            for (int w = 0; w < nw; ++w) s += red[2][w];
+            part[2] = s;
+        }
+        cl.sync();
+    }
+    if (rank == 0 && threadIdx.x == 0) {
         if (center) {
             center[2 * imgi] = a0;
             center[2 * imgi + 1] = a1;
         }
-        if (norm) norm[imgi] = s;
+        if (norm) {
+            double s = 0.0;
+            for (int r = 0; r < S; ++r) s += cl.map_shared_rank(part, r)[2];
+            norm[imgi] = s;
+        }
     }
+    cl.sync();  // no CTA leaves while its sums may still be read
 }
 
 }  // namespace
@@ -582,8 +615,21 @@ cudaError_t launch_center_norm(const float *q, int nb, int n, int M, const doubl
                                double *center, double *norm, cudaStream_t st)
 {
     if (nb <= 0) return cudaSuccess;
-    k_center_norm<<<nb, 256, 0, st>>>(q, n, M, cs64, center, norm);
-    return cudaGetLastError();
+    // CTAs per image: enough for four on each of 152 SMs, eight (the portable
+    // cluster size) at most
+    int S = 1;
+    while (S < 8 && (long long)nb * S < 4 * 152) S *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(nb * S));
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)S;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_center_norm, q, n, M, cs64, center, norm);
 }
 
 }  // namespace swk
