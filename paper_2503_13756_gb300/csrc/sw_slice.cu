@@ -59,16 +59,29 @@
 // exact band-limited projection, at the level of FP32 rounding.
 #include <algorithm>
 
+#include <cooperative_groups.h>
+
 #include "sw_internal.cuh"
 
 namespace swk {
 namespace {
+
+namespace cg = cooperative_groups;
 
 constexpr int kSliceThreads = 1024;  // shared-memory grid: 32 warps
 constexpr int kBigThreads = 512;     // global grid: 16 warps (more registers per lane)
 constexpr int kBigBatch = 32;        // angles per CTA of k_slice_rows
 static_assert(2 * (kSliceThreads / 32) == kSliceBatch, "one warp per angle pair of a batch");
 static_assert(2 * (kBigThreads / 32) == kBigBatch, "one warp per angle pair of a batch");
+
+// Barrier of the CTAs that share an image: the block, or its cluster (which
+// also orders their shared- and global-memory accesses).
+template <bool CL>
+__device__ __forceinline__ void image_sync()
+{
+    if constexpr (CL) cg::this_cluster().sync();
+    else __syncthreads();
+}
 
 // x mod N for the small excursions of the grid indices (|x| < 2N).
 __device__ __forceinline__ int wrap_n(int x, int N)
@@ -138,8 +151,6 @@ __device__ __forceinline__ const float *image_of(const SliceArgs &A, int gi)
     return gi < A.nb1 ? A.img + (size_t)gi * sz : A.img2 + (size_t)(gi - A.nb1) * sz;
 }
 
-// Phases A and B for one image into the grid G (shared or global memory),
-// by nw warps; returns the image's bad/mass flags of this thread.
 __device__ __forceinline__ void cp_async4z(float *dst, const float *src, int src_bytes)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
@@ -154,11 +165,25 @@ __device__ __forceinline__ void cp_async4z(float *dst, const float *src, int src
 // upsampling the image passes through it in 32-column bands by cp.async,
 // band b + 1 in flight while the warps transform band b (one column pair
 // each); otherwise each lane loads its pixels directly.
-template <int M>
+//
+// CL: the CTAs of a cluster share the image: each takes every P-th column
+// pair (or band) and kept row, and the cluster's barrier separates the
+// phases.  With the grid in shared memory (SHARED) a column value goes to the
+// CTA that transforms its row, and finished rows are copied to all CTAs
+// (coalesced: storing every value into every CTA as it was made took longer
+// than one CTA building the whole grid).
+template <int M, bool CL = false, bool SHARED = true>
 __device__ __forceinline__ void slice_grid(const SliceArgs &A, const float *__restrict__ src,
                                            float2 *G, const float2 *tw, int warp, int nw,
                                            int lane, int &bad, int &mass, float *stage = nullptr)
 {
+    const int P = CL ? (int)cg::this_cluster().num_blocks() : 1;
+    const int rank = CL ? (int)cg::this_cluster().block_rank() : 0;
+    // phase A's value of a kept row: to the CTA that transforms the row
+    auto put_row = [&](int i, int idx, float2 val) {
+        if constexpr (CL && SHARED) cg::this_cluster().map_shared_rank(G, i & (P - 1))[idx] = val;
+        else G[idx] = val;
+    };
     constexpr int N = 32 * M;
     const int L = A.L, half = L / 2;
     const int rows = slice_rows(N), S = slice_stride(N), lo = slice_lo(N);
@@ -204,9 +229,10 @@ __device__ __forceinline__ void slice_grid(const SliceArgs &A, const float *__re
             const int i = wrap_n(k1 + kb - lo, N);  // kept row of l2 = kout (mod N)
             if (i < rows) {
                 // column c: (Z + conj Z(-l2)) / 2; column c + 1: (Z - conj Z(-l2)) / (2i)
-                G[i * S + c] = make_float2(0.5f * (Z.x + Zc.x), 0.5f * (Z.y + Zc.y));
+                put_row(i, i * S + c, make_float2(0.5f * (Z.x + Zc.x), 0.5f * (Z.y + Zc.y)));
                 if (c + 1 < L)
-                    G[i * S + c + 1] = make_float2(0.5f * (Z.y - Zc.y), -0.5f * (Z.x - Zc.x));
+                    put_row(i, i * S + c + 1,
+                            make_float2(0.5f * (Z.y - Zc.y), -0.5f * (Z.x - Zc.x)));
             }
         }
     };
@@ -222,13 +248,15 @@ __device__ __forceinline__ void slice_grid(const SliceArgs &A, const float *__re
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
-        issue(0, stage);
-        for (int b = 0; b < nbands; ++b) {
-            if (b + 1 < nbands) issue(b + 1, stage + ((b + 1) & 1) * L * RSB);
+        // buffers in the order of this CTA's bands (rank, rank + P, ...)
+        float *buf0 = stage, *buf1 = stage + L * RSB;
+        if (rank < nbands) issue(rank, buf0);
+        for (int b = rank; b < nbands; b += P) {
+            if (b + P < nbands) issue(b + P, buf1);
             else asm volatile("cp.async.commit_group;" ::: "memory");
             asm volatile("cp.async.wait_group 1;" ::: "memory");
             __syncthreads();
-            const float *buf = stage + (b & 1) * L * RSB;
+            const float *buf = buf0;
             const int c = b * BW + 2 * warp;
             if (c < L)
                 column_pair(c, [&](int r) {
@@ -236,12 +264,15 @@ __device__ __forceinline__ void slice_grid(const SliceArgs &A, const float *__re
                     return make_float2(row[0], c + 1 < L ? row[1] : 0.f);
                 });
             __syncthreads();  // the band's buffer is refilled two bands on
+            float *const nb = buf0;
+            buf0 = buf1;
+            buf1 = nb;
         }
     } else {
         // 8-byte pixel pairs: L even (every row starts 8-byte aligned, c is
         // even) and the image itself 8-byte aligned
         const bool pair8 = (L & 1) == 0 && (reinterpret_cast<uintptr_t>(src) & 7) == 0;
-        for (int c = 2 * warp; c < L; c += 2 * nw)
+        for (int c = 2 * (rank + P * warp); c < L; c += 2 * P * nw)
             column_pair(c, [&](int r) {
                 if (A.srcL == L && pair8) {
                     // (c, c + 1) in one 8-byte load: each lane reads another
@@ -257,9 +288,9 @@ __device__ __forceinline__ void slice_grid(const SliceArgs &A, const float *__re
                 return make_float2(x0, c + 1 < L ? x0 : 0.f);
             });
     }
-    __syncthreads();
+    image_sync<CL>();
     // ---- B: one warp per kept row: FFT along c', left and right columns
-    for (int i = warp; i < rows; i += nw) {
+    for (int i = rank + P * warp; i < rows; i += P * nw) {
         float2 v[M];
 #pragma unroll
         for (int n1 = 0; n1 < M; ++n1) {
@@ -276,6 +307,13 @@ __device__ __forceinline__ void slice_grid(const SliceArgs &A, const float *__re
             const int q = wrap_n(kout - lo, N);  // left column with l1 = kout (mod N)
             if (q < nleft) G[i * S + q] = v[k1];
             if (kout >= 1 && kout <= nright) G[i * S + nleft + nright - kout] = v[k1];
+        }
+        if constexpr (CL && SHARED) {  // the finished row to the other CTAs, coalesced
+            __syncwarp();
+            for (int r = 1; r < P; ++r) {
+                float2 *Gr = cg::this_cluster().map_shared_rank(G, (rank + r) & (P - 1));
+                for (int x = lane; x < nleft + nright; x += 32) Gr[i * S + x] = G[i * S + x];
+            }
         }
     }
 }
@@ -497,29 +535,29 @@ __device__ __forceinline__ void slice_pair(const SliceArgs &A, const float2 *G, 
 // An entry with kSlicePairBit set computes the pair (j, j + 1).  UP: G is
 // the grid of an image of side L/2 (N = 32 M = B/2 points), the samples
 // j <= N those of its 2 x 2 upsampled image (slice_target_up).
-template <int M, int BATCH, bool UP = false>
+// CL: the P CTAs of the cluster take P batches (from batch bi) together, as
+// each inverts only BATCH / P angle rows of a batch: its Xs holds those of
+// all P batches, and the samples go to the shared memory of the CTA that
+// inverts them.
+template <int M, int BATCH, bool UP = false, bool CL = false>
 __device__ __forceinline__ void slice_samples(const SliceArgs &A, const float2 *G, float2 *Xs,
-                                              int k0, int bi)
+                                              int bi)
 {
     constexpr int N = 32 * M;
     const int nh = A.nh;
     const int S = slice_stride(N);
     const int nj = (UP ? N : N / 2) + 1;
-    // rows of angles beyond nh (last batch) read as zero
-    for (int it = threadIdx.x + (nh - k0) * nj; it < BATCH * nj; it += blockDim.x)
-        Xs[it] = make_float2(0.f, 0.f);
-    const int g0 = __ldg(A.goff + bi), ng = __ldg(A.goff + bi + 1) - g0;
-    for (int slot = threadIdx.x; slot < ng * 16; slot += blockDim.x) {
-        const unsigned ent = __ldg(A.gtab + (size_t)(g0 + (slot >> 4)) * 16 + (slot & 15));
-        if (ent == 0xFFFFu) continue;
+    // entry of the table: the samples (k, j), k = k0 + kk, into row(kk)[j]
+    auto entry = [&](unsigned ent, int k0, auto row) {
         const int kk = (int)((ent >> 8) & 63u), j = (int)(ent & 255u);
         const int k = k0 + kk;
         if (ent & kSlicePairBit) {
             float2 xa, xb;
             slice_pair<M, UP>(A, G, S, k, j, xa, xb);
-            Xs[kk * nj + j] = xa;
-            Xs[kk * nj + j + 1] = xb;
-            continue;
+            float2 *X = row(kk);
+            X[j] = xa;
+            X[j + 1] = xb;
+            return;
         }
         float wx[kSliceW], wy[kSliceW];
         int row0, col0;
@@ -530,14 +568,57 @@ __device__ __forceinline__ void slice_samples(const SliceArgs &A, const float2 *
         if (conj) fc.y = -fc.y;
         float2 x = slice_sum(G + row0 * S + col0, S, left ? 1 : -1, wx, wy, fc);
         if (conj) x.y = -x.y;
-        Xs[kk * nj + j] = x;
+        row(kk)[j] = x;
+    };
+    if constexpr (CL) {
+        const int P = (int)cg::this_cluster().num_blocks(), SH = BATCH / P;
+        const int rank = (int)cg::this_cluster().block_rank();
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+        // rows of angles beyond nh read as zero
+        for (int lr = warp; lr < BATCH; lr += nw)
+            if ((bi + lr / SH) * BATCH + rank * SH + lr % SH >= nh)
+                for (int j = lane; j < nj; j += 32) Xs[lr * nj + j] = make_float2(0.f, 0.f);
+        // one warp per two groups, batch after batch (a batch's groups start
+        // a warp: its pair groups are of one pattern per warp)
+        const int bend = min(bi + P, (nh + BATCH - 1) / BATCH);
+        int b = bi, task = rank + P * warp;
+        int g0 = __ldg(A.goff + b), g1 = __ldg(A.goff + b + 1);
+        for (;;) {
+            while (b < bend && 2 * task >= g1 - g0) {
+                task -= (g1 - g0 + 1) / 2;
+                if (++b < bend) {
+                    g0 = g1;
+                    g1 = __ldg(A.goff + b + 1);
+                }
+            }
+            if (b >= bend) break;
+            const int g = g0 + 2 * task + (lane >> 4);
+            const unsigned ent = g < g1 ? __ldg(A.gtab + (size_t)g * 16 + (lane & 15)) : 0xFFFFu;
+            if (ent != 0xFFFFu)
+                entry(ent, b * BATCH, [&](int kk) {
+                    return cg::this_cluster().map_shared_rank(Xs, kk / SH) +
+                           ((b - bi) * SH + kk % SH) * nj;
+                });
+            task += P * nw;
+        }
+    } else {
+        const int k0 = bi * BATCH;
+        // rows of angles beyond nh (last batch) read as zero
+        for (int it = threadIdx.x + (nh - k0) * nj; it < BATCH * nj; it += blockDim.x)
+            Xs[it] = make_float2(0.f, 0.f);
+        const int g0 = __ldg(A.goff + bi), ng = __ldg(A.goff + bi + 1) - g0;
+        for (int slot = threadIdx.x; slot < ng * 16; slot += blockDim.x) {
+            const unsigned ent = __ldg(A.gtab + (size_t)(g0 + (slot >> 4)) * 16 + (slot & 15));
+            if (ent != 0xFFFFu) entry(ent, k0, [&](int kk) { return Xs + kk * nj; });
+        }
     }
-    __syncthreads();
+    image_sync<CL>();
 }
 
 // Phase D for the angles [k0, k0 + BATCH) of image gi from the slice samples
 // Xs; tw in shared memory; BATCH / 2 warps.  Ends with a block barrier.
-template <int M, int BATCH>
+// CL: this CTA's rows of P batches from the one at k0 (slice_samples).
+template <int M, int BATCH, bool CL = false>
 __device__ __forceinline__ void slice_rows_out(const SliceArgs &A, float2 *Xs, const float2 *tw,
                                                int gi, int k0, int warp, int lane)
 {
@@ -547,12 +628,17 @@ __device__ __forceinline__ void slice_rows_out(const SliceArgs &A, float2 *Xs, c
     const float invB = 1.f / (float)N;
     const int nrow = A.full_n ? 2 * nh : nh;
     float *outi = A.out + (size_t)gi * nrow * N;
-    // D: warp w inverse-transforms the angles ka = 2w, kb = 2w + 1 of the
-    // batch as Y_j = X_a + i X_b, Y_{B-j} = conj X_a + i conj X_b
-    // (Y_0, Y_{B/2}: real parts), then writes both rows
-    const int ka = 2 * warp;
-    if (ka < BATCH && k0 + ka < nh) {
-        const float2 *Xa = Xs + ka * nj, *Xb = Xa + nj;
+    // D: warp w inverse-transforms the rows 2w, 2w + 1, angles ka, kb = ka + 1,
+    // as Y_j = X_a + i X_b, Y_{B-j} = conj X_a + i conj X_b (Y_0, Y_{B/2}:
+    // real parts), then writes both rows
+    const int row = 2 * warp;
+    int ka = k0 + row;
+    if constexpr (CL) {
+        const int SH = BATCH / (int)cg::this_cluster().num_blocks();
+        ka = k0 + row / SH * BATCH + (int)cg::this_cluster().block_rank() * SH + row % SH;
+    }
+    if (row < BATCH && ka < nh) {
+        const float2 *Xa = Xs + row * nj, *Xb = Xa + nj;
         float2 v[M];
 #pragma unroll
         for (int n1 = 0; n1 < M; ++n1) {
@@ -566,7 +652,7 @@ __device__ __forceinline__ void slice_rows_out(const SliceArgs &A, float2 *Xs, c
         __syncwarp();
         warp_ifft<M>(v, tw, lane);
         // stage the two rows in this warp's own sample rows (2 nj >= B + 2)
-        float *stw = reinterpret_cast<float *>(Xs + ka * nj);
+        float *stw = reinterpret_cast<float *>(Xs + row * nj);
         const int kb = M * brev5(lane);
 #pragma unroll
         for (int k1 = 0; k1 < M; ++k1) {
@@ -576,7 +662,7 @@ __device__ __forceinline__ void slice_rows_out(const SliceArgs &A, float2 *Xs, c
         __syncwarp();
 #pragma unroll
         for (int h2 = 0; h2 < 2; ++h2) {
-            const int k = k0 + ka + h2;
+            const int k = ka + h2;
             if (k >= nh) break;
             float *o = outi + (size_t)k * N;
             float *om = outi + (size_t)(nh + k) * N + (N - 1);
@@ -588,11 +674,27 @@ __device__ __forceinline__ void slice_rows_out(const SliceArgs &A, float2 *Xs, c
             }
         }
     }
-    __syncthreads();
+    image_sync<CL>();
 }
 
-// L <= 128: one CTA per image, the grid in shared memory.
-template <int M>
+// The image's status from every thread's flags (s_flags: this CTA's word, bit
+// 0 a non-finite pixel, bit 1 positive mass; zeroed before the grid phases).
+template <bool CL>
+__device__ __forceinline__ void image_status(const SliceArgs &A, int gi, int *s_flags, int bad,
+                                             int mass)
+{
+    const int f = (bad ? 1 : 0) | (mass ? 2 : 0);
+    int *dst = s_flags;
+    if constexpr (CL) dst = cg::this_cluster().map_shared_rank(s_flags, 0);
+    if (f) atomicOr(dst, f);
+    image_sync<CL>();
+    if (threadIdx.x == 0 && (!CL || cg::this_cluster().block_rank() == 0))
+        A.status[gi] = *s_flags == 2 ? 0 : 1;
+}
+
+// L <= 128: one CTA, or one cluster of CTAs (CL), per image, the grid in
+// shared memory.
+template <int M, bool CL>
 __global__ void __launch_bounds__(kSliceThreads, 1) k_project_slice(SliceArgs A)
 {
     constexpr int N = 32 * M;
@@ -601,28 +703,25 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_project_slice(SliceArgs A)
     float2 *G = sms;                                        // [rows][S] grid
     float2 *Xs = G + slice_rows(N) * slice_stride(N);       // [kSliceBatch][nj]
     float2 *tw = Xs + kSliceBatch * nj;                     // [N]
-    __shared__ int s_bad, s_mass;
-    const int gi = A.img_off + blockIdx.x;
+    __shared__ int s_flags;
+    const int gi = A.img_off + (CL ? blockIdx.x / cg::this_cluster().num_blocks() : blockIdx.x);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        s_bad = 0;
-        s_mass = 0;
+        s_flags = 0;
         // one CTA per SM: the image that starts about one CTA lifetime from
         // now is pulled into L2, so that its phase-A loads hit there
-        if (A.pf_ahead > 0 && blockIdx.x + A.pf_ahead < gridDim.x)
+        if (!CL && A.pf_ahead > 0 && blockIdx.x + A.pf_ahead < gridDim.x)
             prefetch_l2(image_of(A, gi + A.pf_ahead), sizeof(float) * A.srcL * A.srcL);
     }
     for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = A.tw[i];
-    __syncthreads();
+    image_sync<CL>();
     int bad = 0, mass = 0;
-    slice_grid<M>(A, image_of(A, gi), G, tw, warp, kSliceThreads / 32, lane, bad, mass);
-    if (bad) atomicOr(&s_bad, 1);
-    if (mass) atomicOr(&s_mass, 1);
-    __syncthreads();
-    if (threadIdx.x == 0) A.status[gi] = (s_bad || !s_mass) ? 1 : 0;
-    for (int k0 = 0; k0 < A.nh; k0 += kSliceBatch) {
-        slice_samples<M, kSliceBatch>(A, G, Xs, k0, k0 / kSliceBatch);
-        slice_rows_out<M, kSliceBatch>(A, Xs, tw, gi, k0, warp, lane);
+    slice_grid<M, CL>(A, image_of(A, gi), G, tw, warp, kSliceThreads / 32, lane, bad, mass);
+    image_status<CL>(A, gi, &s_flags, bad, mass);
+    const int step = kSliceBatch * (CL ? (int)cg::this_cluster().num_blocks() : 1);
+    for (int k0 = 0; k0 < A.nh; k0 += step) {
+        slice_samples<M, kSliceBatch, false, CL>(A, G, Xs, k0 / kSliceBatch);
+        slice_rows_out<M, kSliceBatch, CL>(A, Xs, tw, gi, k0, warp, lane);
     }
 }
 
@@ -630,7 +729,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_project_slice(SliceArgs A)
 // grid of the L/2 image (N = 32 MG = B/2 points, A.L = A.srcL = L/2) in
 // shared memory, the slice samples j <= N of the L x L image from it in
 // kUpBatch-angle batches (slice_samples<UP>), and rows of B = 2 N bins.
-template <int MG>
+template <int MG, bool CL>
 __global__ void __launch_bounds__(kSliceThreads, 1) k_project_slice_up(SliceArgs A)
 {
     constexpr int N = 32 * MG;
@@ -640,54 +739,49 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_project_slice_up(SliceArgs
     float2 *Xs = G + slice_rows(N) * slice_stride(N);       // [kUpBatch][nj]
     float2 *tw = Xs + kUpBatch * nj;                        // [N]
     float2 *tw2 = tw + N;                                   // [2 N]
-    __shared__ int s_bad, s_mass;
-    const int gi = A.img_off + blockIdx.x;
+    __shared__ int s_flags;
+    const int gi = A.img_off + (CL ? blockIdx.x / cg::this_cluster().num_blocks() : blockIdx.x);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        s_bad = 0;
-        s_mass = 0;
-        if (A.pf_ahead > 0 && blockIdx.x + A.pf_ahead < gridDim.x)
+        s_flags = 0;
+        if (!CL && A.pf_ahead > 0 && blockIdx.x + A.pf_ahead < gridDim.x)
             prefetch_l2(image_of(A, gi + A.pf_ahead), sizeof(float) * A.srcL * A.srcL);
     }
     for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = A.tw[i];
     for (int i = threadIdx.x; i < 2 * N; i += blockDim.x) tw2[i] = A.tw2[i];
-    __syncthreads();
+    image_sync<CL>();
     int bad = 0, mass = 0;
-    slice_grid<MG>(A, image_of(A, gi), G, tw, warp, kSliceThreads / 32, lane, bad, mass);
-    if (bad) atomicOr(&s_bad, 1);
-    if (mass) atomicOr(&s_mass, 1);
-    __syncthreads();
-    if (threadIdx.x == 0) A.status[gi] = (s_bad || !s_mass) ? 1 : 0;
-    for (int k0 = 0; k0 < A.nh; k0 += kUpBatch) {
-        slice_samples<MG, kUpBatch, true>(A, G, Xs, k0, k0 / kUpBatch);
-        slice_rows_out<2 * MG, kUpBatch>(A, Xs, tw2, gi, k0, warp, lane);
+    slice_grid<MG, CL>(A, image_of(A, gi), G, tw, warp, kSliceThreads / 32, lane, bad, mass);
+    image_status<CL>(A, gi, &s_flags, bad, mass);
+    const int step = kUpBatch * (CL ? (int)cg::this_cluster().num_blocks() : 1);
+    for (int k0 = 0; k0 < A.nh; k0 += step) {
+        slice_samples<MG, kUpBatch, true, CL>(A, G, Xs, k0 / kUpBatch);
+        slice_rows_out<2 * MG, kUpBatch, CL>(A, Xs, tw2, gi, k0, warp, lane);
     }
 }
 
-// 128 < L: the grid of image img_off + blockIdx.x into A.grid[blockIdx.x].
-template <int M>
+// 128 < L: the grid of image img_off + i into A.grid[i], by CTA i or by the
+// CTAs of cluster i (CL).
+template <int M, bool CL>
 __global__ void __launch_bounds__(kBigThreads, 2) k_slice_grid(SliceArgs A)
 {
     constexpr int N = 32 * M;
     __shared__ float2 tw[N];
-    __shared__ int s_bad, s_mass;
-    const int gi = A.img_off + blockIdx.x;
+    __shared__ int s_flags;
+    const int gi = A.img_off + (CL ? blockIdx.x / cg::this_cluster().num_blocks() : blockIdx.x);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        s_bad = 0;
-        s_mass = 0;
+        s_flags = 0;
     }
     for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = A.tw[i];
-    __syncthreads();
+    image_sync<CL>();
     extern __shared__ float stg[];  // [2][L][33] image bands (not upsampled)
-    float2 *G = A.grid + (size_t)blockIdx.x * slice_rows(N) * slice_stride(N);
+    float2 *G = A.grid + (size_t)(gi - A.img_off) * slice_rows(N) * slice_stride(N);
     int bad = 0, mass = 0;
-    slice_grid<M>(A, image_of(A, gi), G, tw, warp, kBigThreads / 32, lane, bad, mass,
-                  A.srcL == A.L ? stg : nullptr);
-    if (bad) atomicOr(&s_bad, 1);
-    if (mass) atomicOr(&s_mass, 1);
-    __syncthreads();
-    if (threadIdx.x == 0) A.status[gi] = (s_bad || !s_mass) ? 1 : 0;
+    slice_grid<M, CL, false>(A, image_of(A, gi), G, tw, warp, kBigThreads / 32, lane, bad, mass,
+                             A.srcL == A.L ? stg : nullptr);
+    image_status<CL>(A, gi, &s_flags, bad, mass);
+    if constexpr (CL) cg::this_cluster().sync();  // the flags' word outlives its writers
 }
 
 // 128 < L: the slice samples whose footprints start in tile blockIdx.x of
@@ -753,34 +847,76 @@ __global__ void __launch_bounds__(kBigThreads, 2) k_slice_rows(SliceArgs A)
                                  threadIdx.x & 31);
 }
 
+// Multiprocessors of the current device.
+cudaError_t sm_count(int *sms)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    return e != cudaSuccess ? e : cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+}
+
+// CTAs per image (a power of two, at most the portable cluster size 8) for nb
+// images where per_sm CTAs fit an SM: the widest cluster with room for all
+// images at once.  A cluster stays within one of the (at least eight) GPCs,
+// so one of 8 is counted against sms / 8 SMs a GPC.
+int cluster_width(int nb, int sms, int per_sm)
+{
+    const int gpc = sms / 8 * per_sm;  // CTA slots of a GPC
+    for (int P = 8; P > 1; P /= 2)
+        if (nb <= 8 * (gpc / P)) return P;
+    return 1;
+}
+
+template <typename K>
+cudaError_t launch_cluster(K kern, int nb, int P, int threads, size_t smem, const SliceArgs &a,
+                           cudaStream_t st)
+{
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(nb * P));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)P;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = P > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+// One CTA per image, or, for fewer images than would fill the chip, a
+// cluster (one CTA holds all the shared memory of its SM).  A pair of 64 x 64
+// images at n = 360: 48 us on two CTAs, 22 us on two clusters of 8; three
+// half-size images at L = 256, n = 360: 174 against 47 us.  With all angle
+// batches in turn, two cluster barriers each, these took 37 and 87 us.
 template <int M>
 cudaError_t launch_small(SliceArgs a, int nb, cudaStream_t st)
 {
-    const size_t smem = slice_smem_bytes(32 * M);
-    cudaError_t e = cudaFuncSetAttribute(k_project_slice<M>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int sms = 0;
+    cudaError_t e = sm_count(&sms);
     if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
-        a.pf_ahead = sms;  // resident CTAs: one per SM
-    k_project_slice<M><<<nb, kSliceThreads, smem, st>>>(a);
-    return cudaGetLastError();
+    a.pf_ahead = sms;  // resident CTAs: one per SM
+    const int P = cluster_width(nb, sms, 1);
+    const size_t smem = slice_smem_bytes(32 * M);
+    return P > 1 ? launch_cluster(k_project_slice<M, true>, nb, P, kSliceThreads, smem, a, st)
+                 : launch_cluster(k_project_slice<M, false>, nb, 1, kSliceThreads, smem, a, st);
 }
 
 template <int MG>
 cudaError_t launch_up(SliceArgs a, int nb, cudaStream_t st)
 {
-    const size_t smem = slice_up_smem_bytes(64 * MG);
-    cudaError_t e = cudaFuncSetAttribute(k_project_slice_up<MG>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int sms = 0;
+    cudaError_t e = sm_count(&sms);
     if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
-        a.pf_ahead = sms;
-    k_project_slice_up<MG><<<nb, kSliceThreads, smem, st>>>(a);
-    return cudaGetLastError();
+    a.pf_ahead = sms;
+    const int P = cluster_width(nb, sms, 1);
+    const size_t smem = slice_up_smem_bytes(64 * MG);
+    return P > 1 ? launch_cluster(k_project_slice_up<MG, true>, nb, P, kSliceThreads, smem, a, st)
+                 : launch_cluster(k_project_slice_up<MG, false>, nb, 1, kSliceThreads, smem, a, st);
 }
 
 template <int M>
@@ -795,9 +931,8 @@ cudaError_t launch_big(SliceArgs a, int nb, int chunk, cudaStream_t st)
     if (e != cudaSuccess) return e;
     // two 32-column bands of the image (rows 33 floats apart) when not upsampled
     const size_t smem_grid = a.srcL == a.L ? sizeof(float) * 2 * (size_t)a.L * 33 : 0;
-    e = cudaFuncSetAttribute(k_slice_grid<M>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem_grid);
-    if (e != cudaSuccess) return e;
+    int sms = 0;
+    if ((e = sm_count(&sms)) != cudaSuccess) return e;
     // chunks of equal size (at most `chunk`): no small last chunk whose
     // launches would leave most SMs idle
     const int nchunks = (nb + chunk - 1) / chunk;
@@ -805,7 +940,10 @@ cudaError_t launch_big(SliceArgs a, int nb, int chunk, cudaStream_t st)
     for (int i0 = 0; i0 < nb; i0 += chunk) {
         const int cnt = std::min(chunk, nb - i0);
         a.img_off = i0;
-        k_slice_grid<M><<<cnt, kBigThreads, smem_grid, st>>>(a);
+        const int P = cluster_width(cnt, sms, 2);
+        e = P > 1 ? launch_cluster(k_slice_grid<M, true>, cnt, P, kBigThreads, smem_grid, a, st)
+                  : launch_cluster(k_slice_grid<M, false>, cnt, 1, kBigThreads, smem_grid, a, st);
+        if (e != cudaSuccess) return e;
         k_slice_tile<M><<<dim3(ntiles, cnt), kBigThreads, 0, st>>>(a);
         k_slice_rows<M><<<dim3(nbatch, cnt), kBigThreads, smem, st>>>(a);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
