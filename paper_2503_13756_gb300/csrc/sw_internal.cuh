@@ -230,6 +230,76 @@ __device__ __forceinline__ void lane_dft(float2 (&v)[M], const float2 *__restric
 // buffer that holds the result.  Must be called by every thread of the block;
 // ends with a __syncthreads().
 
+// R-point butterfly V[m] = sum_i v[i] e^{DIR 2 pi i m i / R}.
+template <int R, int DIR>
+__device__ __forceinline__ void butterfly(const float2 (&v)[R], float2 (&V)[R])
+{
+    if constexpr (R == 2) {
+        V[0] = cadd(v[0], v[1]);
+        V[1] = csub(v[0], v[1]);
+    } else if constexpr (R == 4) {
+        float2 s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]);
+        float2 s13 = cadd(v[1], v[3]), d13 = cmul_i(csub(v[1], v[3]), DIR);
+        V[0] = cadd(s02, s13);
+        V[2] = csub(s02, s13);
+        V[1] = cadd(d02, d13);
+        V[3] = csub(d02, d13);
+    } else if constexpr (R == 3) {
+        // w3 = e^{DIR 2 pi i / 3} = -1/2 + DIR i sqrt(3)/2
+        const float c3 = -0.5f, s3 = 0.86602540378443864676f;
+        float2 t1 = cadd(v[1], v[2]);
+        float2 t2 = make_float2(v[0].x + c3 * t1.x, v[0].y + c3 * t1.y);
+        float2 t3 = cmul_i(csub(v[1], v[2]), DIR);
+        t3.x *= s3;
+        t3.y *= s3;
+        V[0] = cadd(v[0], t1);
+        V[1] = cadd(t2, t3);
+        V[2] = csub(t2, t3);
+    } else if constexpr (R == 8) {
+        // two radix-4 butterflies over the even and the odd inputs, then
+        // V[m] = E[m] + w8^m O[m], V[m+4] = E[m] - w8^m O[m], with
+        // w8 = e^{DIR 2 pi i / 8} = (1 + DIR i) / sqrt(2)
+        const float r2 = 0.70710678118654752440f;
+        float2 E[4], O[4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            float2 e0 = cadd(v[h], v[h + 4]), e1 = csub(v[h], v[h + 4]);
+            float2 e2 = cadd(v[h + 2], v[h + 6]);
+            float2 e3 = cmul_i(csub(v[h + 2], v[h + 6]), DIR);
+            float2 *X = h == 0 ? E : O;
+            X[0] = cadd(e0, e2);
+            X[2] = csub(e0, e2);
+            X[1] = cadd(e1, e3);
+            X[3] = csub(e1, e3);
+        }
+        O[1] = make_float2(r2 * (O[1].x - DIR * O[1].y), r2 * (O[1].y + DIR * O[1].x));
+        O[2] = cmul_i(O[2], DIR);
+        O[3] = make_float2(r2 * (-O[3].x - DIR * O[3].y), r2 * (-O[3].y + DIR * O[3].x));
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            V[m] = cadd(E[m], O[m]);
+            V[m + 4] = csub(E[m], O[m]);
+        }
+    } else {  // R == 5
+        const float c1 = 0.30901699437494742410f;   // cos(2 pi / 5)
+        const float c2 = -0.80901699437494742410f;  // cos(4 pi / 5)
+        const float s1 = 0.95105651629515357212f;   // sin(2 pi / 5)
+        const float s2 = 0.58778525229247312917f;   // sin(4 pi / 5)
+        float2 a1 = cadd(v[1], v[4]), b1 = csub(v[1], v[4]);
+        float2 a2 = cadd(v[2], v[3]), b2 = csub(v[2], v[3]);
+        float2 r1 = make_float2(v[0].x + c1 * a1.x + c2 * a2.x, v[0].y + c1 * a1.y + c2 * a2.y);
+        float2 r2 = make_float2(v[0].x + c2 * a1.x + c1 * a2.x, v[0].y + c2 * a1.y + c1 * a2.y);
+        // i1 = DIR*i*(s1 b1 + s2 b2), i2 = DIR*i*(s2 b1 - s1 b2)
+        float2 i1 = cmul_i(make_float2(s1 * b1.x + s2 * b2.x, s1 * b1.y + s2 * b2.y), DIR);
+        float2 i2 = cmul_i(make_float2(s2 * b1.x - s1 * b2.x, s2 * b1.y - s1 * b2.y), DIR);
+        V[0] = make_float2(v[0].x + a1.x + a2.x, v[0].y + a1.y + a2.y);
+        V[1] = cadd(r1, i1);
+        V[4] = csub(r1, i1);
+        V[2] = cadd(r2, i2);
+        V[3] = csub(r2, i2);
+    }
+}
+
 // One stage of radix R: item t = (j, s) takes x[j + i n/R] (i < R), twiddled
 // by w^{i k}, k = j mod Ns, and writes its R outputs at stride Ns from
 // (j div Ns) Ns R + k.
@@ -257,77 +327,68 @@ __device__ __forceinline__ void fft_stage(const float2 *__restrict__ a, float2 *
             v[i] = x;
         }
         float2 V[R];
-        if (R == 2) {
-            V[0] = cadd(v[0], v[1]);
-            V[1] = csub(v[0], v[1]);
-        } else if (R == 4) {
-            float2 s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]);
-            float2 s13 = cadd(v[1], v[3]), d13 = cmul_i(csub(v[1], v[3]), DIR);
-            V[0] = cadd(s02, s13);
-            V[2] = csub(s02, s13);
-            V[1] = cadd(d02, d13);
-            V[3] = csub(d02, d13);
-        } else if (R == 3) {
-            // w3 = e^{DIR 2 pi i / 3} = -1/2 + DIR i sqrt(3)/2
-            const float c3 = -0.5f, s3 = 0.86602540378443864676f;
-            float2 t1 = cadd(v[1], v[2]);
-            float2 t2 = make_float2(v[0].x + c3 * t1.x, v[0].y + c3 * t1.y);
-            float2 t3 = cmul_i(csub(v[1], v[2]), DIR);
-            t3.x *= s3;
-            t3.y *= s3;
-            V[0] = cadd(v[0], t1);
-            V[1] = cadd(t2, t3);
-            V[2] = csub(t2, t3);
-        } else if (R == 8) {
-            // two radix-4 butterflies over the even and the odd inputs, then
-            // V[m] = E[m] + w8^m O[m], V[m+4] = E[m] - w8^m O[m], with
-            // w8 = e^{DIR 2 pi i / 8} = (1 + DIR i) / sqrt(2)
-            const float r2 = 0.70710678118654752440f;
-            float2 E[4], O[4];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                float2 e0 = cadd(v[h], v[h + 4]), e1 = csub(v[h], v[h + 4]);
-                float2 e2 = cadd(v[h + 2], v[h + 6]);
-                float2 e3 = cmul_i(csub(v[h + 2], v[h + 6]), DIR);
-                float2 *X = h == 0 ? E : O;
-                X[0] = cadd(e0, e2);
-                X[2] = csub(e0, e2);
-                X[1] = cadd(e1, e3);
-                X[3] = csub(e1, e3);
-            }
-            O[1] = make_float2(r2 * (O[1].x - DIR * O[1].y), r2 * (O[1].y + DIR * O[1].x));
-            O[2] = cmul_i(O[2], DIR);
-            O[3] = make_float2(r2 * (-O[3].x - DIR * O[3].y), r2 * (-O[3].y + DIR * O[3].x));
-#pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                V[m] = cadd(E[m], O[m]);
-                V[m + 4] = csub(E[m], O[m]);
-            }
-        } else {  // R == 5
-            const float c1 = 0.30901699437494742410f;   // cos(2 pi / 5)
-            const float c2 = -0.80901699437494742410f;  // cos(4 pi / 5)
-            const float s1 = 0.95105651629515357212f;   // sin(2 pi / 5)
-            const float s2 = 0.58778525229247312917f;   // sin(4 pi / 5)
-            float2 a1 = cadd(v[1], v[4]), b1 = csub(v[1], v[4]);
-            float2 a2 = cadd(v[2], v[3]), b2 = csub(v[2], v[3]);
-            float2 r1 = make_float2(v[0].x + c1 * a1.x + c2 * a2.x, v[0].y + c1 * a1.y + c2 * a2.y);
-            float2 r2 = make_float2(v[0].x + c2 * a1.x + c1 * a2.x, v[0].y + c2 * a1.y + c1 * a2.y);
-            // i1 = DIR*i*(s1 b1 + s2 b2), i2 = DIR*i*(s2 b1 - s1 b2)
-            float2 i1 = cmul_i(make_float2(s1 * b1.x + s2 * b2.x, s1 * b1.y + s2 * b2.y), DIR);
-            float2 i2 = cmul_i(make_float2(s2 * b1.x - s1 * b2.x, s2 * b1.y - s1 * b2.y), DIR);
-            V[0] = make_float2(v[0].x + a1.x + a2.x, v[0].y + a1.y + a2.y);
-            V[1] = cadd(r1, i1);
-            V[4] = csub(r1, i1);
-            V[2] = cadd(r2, i2);
-            V[3] = csub(r2, i2);
-        }
+        butterfly<R, DIR>(v, V);
         const int base = jq * Ns * R + k;
 #pragma unroll
         for (int i = 0; i < R; ++i) b[(base + i * Ns) * NSIG + s] = V[i];
     }
 }
 
-template <int NSIG, int DIR>
+// Two stages of radices R1 (span Ns) and R2 (span Ns R1) in one pass over
+// shared memory, R1 R2 values in registers: with T = n / (R1 R2), item (j, s),
+// j < T, runs the R2 first-stage butterflies j + T i, which share their
+// twiddles and whose m-th outputs are the inputs of the second-stage butterfly
+// (j div Ns) Ns R1 + j mod Ns + m Ns.  The same operations on every value as
+// two calls of fft_stage (a factor e^0 = 1 is multiplied where Ns > 1), half
+// of the passes, block barriers and index arithmetic.
+template <int R1, int R2, int NSIG, int DIR>
+__device__ __forceinline__ void fft_stage2(const float2 *__restrict__ a, float2 *__restrict__ b,
+                                           int n, int Ns, unsigned rcp, int tstep1, int tstep2,
+                                           const float2 *__restrict__ tw)
+{
+    const int T = n / (R1 * R2), nr = n / R1;
+    const int total = T * NSIG;
+    auto twiddle = [&](float2 x, int idx) {
+        float2 w = tw[idx];
+        if (DIR > 0) w.y = -w.y;
+        return cmul(x, w);
+    };
+    for (int t = threadIdx.x; t < total; t += blockDim.x) {
+        const int s = t % NSIG;
+        const int j = t / NSIG;
+        const int jq = Ns == 1 ? j : (int)__umulhi((unsigned)j, rcp);  // j / Ns
+        const int k = j - jq * Ns;
+        float2 y[R1][R2];
+#pragma unroll
+        for (int i = 0; i < R2; ++i) {
+            float2 v[R1], V[R1];
+#pragma unroll
+            for (int m = 0; m < R1; ++m) {
+                v[m] = a[(j + T * i + m * nr) * NSIG + s];
+                if (m > 0 && Ns > 1) v[m] = twiddle(v[m], m * k * tstep1);
+            }
+            butterfly<R1, DIR>(v, V);
+#pragma unroll
+            for (int m = 0; m < R1; ++m) y[m][i] = V[m];
+        }
+        const int base = jq * Ns * R1 * R2 + k;
+#pragma unroll
+        for (int m = 0; m < R1; ++m) {
+            const int k2 = k + m * Ns;
+            float2 V[R2];
+#pragma unroll
+            for (int i = 1; i < R2; ++i)
+                if (m > 0 || Ns > 1) y[m][i] = twiddle(y[m][i], i * k2 * tstep2);
+            butterfly<R2, DIR>(y[m], V);
+#pragma unroll
+            for (int i = 0; i < R2; ++i) b[(base + m * Ns + i * Ns * R1) * NSIG + s] = V[i];
+        }
+    }
+}
+
+// FUSE: stages in pairs where fft_stage2 is built for them (the pairs of the
+// default plans; R1 R2 complex values in registers).
+template <int NSIG, int DIR, bool FUSE = false>
 __device__ __forceinline__ float2 *fft_smem(float2 *a, float2 *b, const FftPlan &plan,
                                             const float2 *tw)
 {
@@ -336,12 +397,31 @@ __device__ __forceinline__ float2 *fft_smem(float2 *a, float2 *b, const FftPlan 
         const int Ns = plan.ns[st];
         const unsigned rcp = plan.ns_rcp[st];
         const int tstep = plan.tstep[st];
-        switch (plan.radix[st]) {
-        case 4: fft_stage<4, NSIG, DIR>(a, b, n, Ns, rcp, tstep, tw); break;
-        case 8: fft_stage<8, NSIG, DIR>(a, b, n, Ns, rcp, tstep, tw); break;
-        case 2: fft_stage<2, NSIG, DIR>(a, b, n, Ns, rcp, tstep, tw); break;
-        case 3: fft_stage<3, NSIG, DIR>(a, b, n, Ns, rcp, tstep, tw); break;
-        default: fft_stage<5, NSIG, DIR>(a, b, n, Ns, rcp, tstep, tw); break;
+        bool two = false;
+        if constexpr (FUSE) {
+            if (st + 1 < plan.nst) {
+                const int t2 = plan.tstep[st + 1];
+                two = true;
+                switch (plan.radix[st] * 10 + plan.radix[st + 1]) {
+                case 44: fft_stage2<4, 4, NSIG, DIR>(a, b, n, Ns, rcp, tstep, t2, tw); break;
+                case 42: fft_stage2<4, 2, NSIG, DIR>(a, b, n, Ns, rcp, tstep, t2, tw); break;
+                case 43: fft_stage2<4, 3, NSIG, DIR>(a, b, n, Ns, rcp, tstep, t2, tw); break;
+                case 23: fft_stage2<2, 3, NSIG, DIR>(a, b, n, Ns, rcp, tstep, t2, tw); break;
+                case 33: fft_stage2<3, 3, NSIG, DIR>(a, b, n, Ns, rcp, tstep, t2, tw); break;
+                case 35: fft_stage2<3, 5, NSIG, DIR>(a, b, n, Ns, rcp, tstep, t2, tw); break;
+                default: two = false;
+                }
+                if (two) ++st;
+            }
+        }
+        if (!two) {
+            switch (plan.radix[st]) {
+            case 4: fft_stage<4, NSIG, DIR>(a, b, n, Ns, rcp, tstep, tw); break;
+            case 8: fft_stage<8, NSIG, DIR>(a, b, n, Ns, rcp, tstep, tw); break;
+            case 2: fft_stage<2, NSIG, DIR>(a, b, n, Ns, rcp, tstep, tw); break;
+            case 3: fft_stage<3, NSIG, DIR>(a, b, n, Ns, rcp, tstep, tw); break;
+            default: fft_stage<5, NSIG, DIR>(a, b, n, Ns, rcp, tstep, tw); break;
+            }
         }
         __syncthreads();
         float2 *tmp = a;

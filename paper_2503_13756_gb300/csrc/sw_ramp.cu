@@ -24,7 +24,7 @@ constexpr int kRampThreads = 256;
 #endif
 
 template <int nsig>
-__global__ void __launch_bounds__(kRampThreads)
+__global__ void __launch_bounds__(kRampThreads, 4)
 k_ramp(const float *__restrict__ proj, int nh, int B, FftPlan plan,
        const float2 *__restrict__ tw, float *__restrict__ parts)
 {
@@ -54,7 +54,7 @@ k_ramp(const float *__restrict__ proj, int nh, int B, FftPlan plan,
             b0[t] = make_float2(tile[(2 * sg) * TS + b], tile[(2 * sg + 1) * TS + b]);
         }
         __syncthreads();
-        float2 *X = fft_smem<nsig, -1>(b0, b1, plan, tws);
+        float2 *X = fft_smem<nsig, -1, true>(b0, b1, plan, tws);
         float2 *Y = X == b0 ? b1 : b0;
         for (int t = threadIdx.x; t < B * nsig; t += blockDim.x) {
             const int j = t / nsig;
@@ -62,7 +62,7 @@ k_ramp(const float *__restrict__ proj, int nh, int B, FftPlan plan,
             X[t] = make_float2(w * X[t].x, w * X[t].y);
         }
         __syncthreads();
-        const float2 *R = fft_smem<nsig, +1>(X, Y, plan, tws);
+        const float2 *R = fft_smem<nsig, +1, true>(X, Y, plan, tws);
         // ---- unpack to rows, then split and write (coalesced)
         for (int t = threadIdx.x; t < B * nsig; t += blockDim.x) {
             const int b = t / nsig, sg = t % nsig;

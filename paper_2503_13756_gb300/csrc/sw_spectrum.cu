@@ -116,20 +116,20 @@ __device__ __forceinline__ void emit(const SpecOut &o, int img, int M, int kf, i
     }
 }
 
+// Two values as one packed pair of the type, and back.
 template <typename T>
 struct Pair2;
 template <>
 struct Pair2<__half> {
     using V = __half2;
-    static __device__ __forceinline__ V make(__half a, __half b) { return __halves2half2(a, b); }
+    static __device__ __forceinline__ V pack(float a, float b) { return __floats2half2_rn(a, b); }
+    static __device__ __forceinline__ float2 unpack(V v) { return __half22float2(v); }
 };
 template <>
 struct Pair2<__nv_bfloat16> {
     using V = __nv_bfloat162;
-    static __device__ __forceinline__ V make(__nv_bfloat16 a, __nv_bfloat16 b)
-    {
-        return __halves2bfloat162(a, b);
-    }
+    static __device__ __forceinline__ V pack(float a, float b) { return __floats2bfloat162_rn(a, b); }
+    static __device__ __forceinline__ float2 unpack(V v) { return __bfloat1622float2(v); }
 };
 
 // emit for the two levels pa (even) and pa + 1 of one frequency at once, M
@@ -149,9 +149,8 @@ __device__ __forceinline__ void emit2(const SpecOut &o, int img, int M, int kf, 
     }
     using P = Pair2<T>;
     using V = typename P::V;
-    const T rea = to_lp<T>(Xa.x), ima = to_lp<T>(Xa.y), reb = to_lp<T>(Xb.x), imb = to_lp<T>(Xb.y);
-    const float rfa = from_lp<T>(rea), imfa = from_lp<T>(ima);
-    const float rfb = from_lp<T>(reb), imfb = from_lp<T>(imb);
+    const V re2 = P::pack(Xa.x, Xb.x), im2 = P::pack(Xa.y, Xb.y);  // (pa, pa + 1)
+    const float2 rf = P::unpack(re2), imf = P::unpack(im2);
     const bool tmpl = img >= o.Nq;
     const int seg = o.ldk;
     const int row_len = o.split ? 2 * seg : seg;
@@ -160,32 +159,29 @@ __device__ __forceinline__ void emit2(const SpecOut &o, int img, int M, int kf, 
                 : reinterpret_cast<T *>(o.lp_q) + (size_t)(kf - 1) * o.lpq_fstride +
                       (size_t)img * row_len;
     auto put = [](T *dst, V v) { *reinterpret_cast<V *>(dst) = v; };
-    const V re2 = P::make(rea, reb), im2 = P::make(ima, imb);
-    const V nim2 = P::make(to_lp<T>(-imfa), to_lp<T>(-imfb));
     if (!o.split) {
-        kahan_add(acc16, w * fmaf(rfa, rfa, imfa * imfa));
-        kahan_add(acc16, w * fmaf(rfb, rfb, imfb * imfb));
+        kahan_add(acc16, w * fmaf(rf.x, rf.x, imf.x * imf.x));
+        kahan_add(acc16, w * fmaf(rf.y, rf.y, imf.y * imf.y));
         put(r + pa, re2);
         put(r + M + pa, im2);
         if (tmpl) {
-            put(r + row_len + pa, nim2);  // row 2j+1: [ -im | re | 0 ]
+            put(r + row_len + pa, __hneg2(im2));  // row 2j+1: [ -im | re | 0 ]
             put(r + row_len + M + pa, re2);
         }
         return;
     }
     // FP16 split: lo = x - hi, exact in FP32, rounded to FP16
-    const V rel2 = P::make(to_lp<T>(Xa.x - rfa), to_lp<T>(Xb.x - rfb));
-    const V iml2 = P::make(to_lp<T>(Xa.y - imfa), to_lp<T>(Xb.y - imfb));
+    const V rel2 = P::pack(Xa.x - rf.x, Xb.x - rf.y);
+    const V iml2 = P::pack(Xa.y - imf.x, Xb.y - imf.y);
     put(r + pa, re2);  // [hi | lo]
     put(r + M + pa, im2);
     put(r + seg + pa, rel2);
     put(r + seg + M + pa, iml2);
-    if (tmpl) {  // row 2j+1: [-im | re]
-        const V nrel2 = P::make(to_lp<T>(-(Xa.y - imfa)), to_lp<T>(-(Xb.y - imfb)));
+    if (tmpl) {  // row 2j+1: [-im | re] (rounding is symmetric)
         T *r2 = r + row_len;
-        put(r2 + pa, nim2);
+        put(r2 + pa, __hneg2(im2));
         put(r2 + M + pa, re2);
-        put(r2 + seg + pa, nrel2);
+        put(r2 + seg + pa, __hneg2(iml2));
         put(r2 + seg + M + pa, rel2);
     }
 }
@@ -207,19 +203,23 @@ __device__ __forceinline__ void cpa4(void *dst, const void *src, int src_bytes)
 
 // Issue the copies of the level batch [p0, p0 + 2 nsig) of image qi into
 // buf: signal s of angle k is buf[k nsig + s] = (level p0 + 2s, p0 + 2s + 1);
-// levels past M are zero-filled.  With one part and M % 4 == 0 every angle's
-// slice is whole 16-byte chunks; otherwise one 4-byte copy per level.
+// levels past M are zero-filled.  With whole groups of four levels per part
+// every angle's slice is 16-byte chunks, each within one part; otherwise one
+// 4-byte copy per level.
 template <int nsig>
 __device__ __forceinline__ void stage_levels(const float *__restrict__ qi, int n, int M, int Mp,
                                              int parts, int p0, float2 *buf)
 {
-    if (parts == 1 && (M & 3) == 0) {
+    if ((Mp & 3) == 0) {
         constexpr int CH = nsig / 2;  // 16-byte chunks (4 levels) per angle
         for (int c = threadIdx.x; c < n * CH; c += blockDim.x) {
             const int k = c / CH, h = c % CH;
             const int p = p0 + 4 * h;
             const int valid = min(max(M - p, 0), 4);
-            const float *src = valid ? qi + (size_t)k * M + p : qi;
+            // level p of part p / Mp (the parts' arrays lie one after the other)
+            const bool second = parts == 2 && p >= Mp;
+            const float *src = valid ? qi + (size_t)(second ? n + k : k) * Mp + (second ? p - Mp : p)
+                                     : qi;
             cpa16(buf + k * nsig + 2 * h, src, 4 * valid);
         }
     } else {
@@ -237,7 +237,7 @@ __device__ __forceinline__ void stage_levels(const float *__restrict__ qi, int n
 }
 
 template <typename T, int nsig>
-__global__ void __launch_bounds__(kSpecThreads)
+__global__ void __launch_bounds__(kSpecThreads, 3)
 k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2 *__restrict__ tw,
            SpecOut o, float *__restrict__ prof, double *__restrict__ center,
            double *__restrict__ norm32, double *__restrict__ norm16, int parts)
@@ -272,7 +272,7 @@ k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2
         // ---- batch: levels (p0 + 2s, p0 + 2s + 1) as signal s (re, im)
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncthreads();
-        float2 *R = fft_smem<nsig, -1>(cur, oth, plan, tws);
+        float2 *R = fft_smem<nsig, -1, true>(cur, oth, plan, tws);
         // the next batch goes to the buffer the transform did not end in
         // (fft_smem ends with a block barrier: both buffers' readers are done)
         float2 *nxt = R == cur ? oth : cur;
@@ -283,7 +283,7 @@ k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2
         for (int t = threadIdx.x; t < (nh + 1) * nsig; t += blockDim.x) {
             const int kf = t / nsig, s = t % nsig;
             const float2 Z = R[kf * nsig + s];
-            const float2 Zc = cconj(R[((n - kf) % n) * nsig + s]);
+            const float2 Zc = cconj(R[(kf ? n - kf : 0) * nsig + s]);
             // Xa = (Z + conj Z(n-k))/2, Xb = (Z - conj Z(n-k)) / (2i)
             const float2 Xa = make_float2(0.5f * (Z.x + Zc.x), 0.5f * (Z.y + Zc.y));
             const float2 dz = make_float2(0.5f * (Z.x - Zc.x), 0.5f * (Z.y - Zc.y));
