@@ -16,19 +16,24 @@
 // real levels packed into one complex signal, FFT'd by the shared-memory
 // Stockham FFT and unpacked by Hermitian symmetry.  The batches are staged
 // by cp.async into two buffers, so that batch b + 1 is in flight while batch
-// b is transformed and written.  Norms are accumulated in double-float.
+// b is transformed and written.  Norms are compensated FP32 sums.
 // Optional BF16/FP16 copies feed the tensor-core GEMM, with their norms taken
 // from the rounded values so that self-distances cancel.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
+
+#include <algorithm>
 
 #include "sw_internal.cuh"
 
 namespace swk {
 namespace {
 
+namespace cg = cooperative_groups;
+
 constexpr int kSpecThreads = 256;
-constexpr size_t kSmemOptIn = 227 * 1024;  // dynamic shared memory a CTA may opt in to
+constexpr size_t kSmemOptIn = 227 * 1024 - 512;  // dynamic shared memory of a CTA, beside the static
 
 template <typename T>
 __device__ __forceinline__ T to_lp(float x);
@@ -66,18 +71,19 @@ __device__ __forceinline__ void kahan_add(DF &a, float x)
     a.hi = t;
 }
 
-// Writes Qhat(kf, p) (kf >= 1) for image img and adds its |.|^2 (weight w)
-// to acc32 (FP32 values) and acc16 (the low-precision values the GEMM sees).
+// Writes Qhat(kf, p) (kf >= 1) for image img and returns its |.|^2 (weight w)
+// for the norm: of the low-precision values where the GEMM sees only those
+// (BF16, FP16), of the FP32 values otherwise.
 template <typename T>
-__device__ __forceinline__ void emit(const SpecOut &o, int img, int M, int kf, int p, float2 X,
-                                     float w, DF &acc32, DF &acc16)
+__device__ __forceinline__ float emit(const SpecOut &o, int img, int M, int kf, int p, float2 X,
+                                      float w)
 {
-    kahan_add(acc32, w * fmaf(X.x, X.x, X.y * X.y));
+    const float term = w * fmaf(X.x, X.x, X.y * X.y);
     if (!o.lp) {
         float *row = o.spec32 + (size_t)(kf - 1) * o.fstride + (size_t)img * 2 * M;
         row[p] = X.x;
         row[M + p] = X.y;
-        return;
+        return term;
     }
     const T re = to_lp<T>(X.x), im = to_lp<T>(X.y);
     const float rf = from_lp<T>(re), imf = from_lp<T>(im);
@@ -90,14 +96,13 @@ __device__ __forceinline__ void emit(const SpecOut &o, int img, int M, int kf, i
                 : reinterpret_cast<T *>(o.lp_q) + (size_t)(kf - 1) * o.lpq_fstride +
                       (size_t)img * row_len;
     if (!o.split) {
-        kahan_add(acc16, w * fmaf(rf, rf, imf * imf));
         r[p] = re;
         r[M + p] = im;
         if (tmpl) {
             r[row_len + p] = nim;  // row 2j+1: [ -im | re | 0 ]
             r[row_len + M + p] = re;
         }
-        return;
+        return w * fmaf(rf, rf, imf * imf);
     }
     // FP16 split: lo = x - hi, exact in FP32, rounded to FP16; rows [hi | lo]
     // (the correlation reads segments hi hi, hi lo, lo hi of its operands)
@@ -114,6 +119,7 @@ __device__ __forceinline__ void emit(const SpecOut &o, int img, int M, int kf, i
         r2[seg + p] = nrel;
         r2[seg + M + p] = rel;
     }
+    return term;
 }
 
 // Two values as one packed pair of the type, and back.
@@ -136,16 +142,16 @@ struct Pair2<__nv_bfloat16> {
 // even: every row segment then takes the pair as one 4-byte store (FP32
 // rows: one 8-byte store), the same values as two emit calls.
 template <typename T>
-__device__ __forceinline__ void emit2(const SpecOut &o, int img, int M, int kf, int pa, float2 Xa,
-                                      float2 Xb, float w, DF &acc32, DF &acc16)
+__device__ __forceinline__ float2 emit2(const SpecOut &o, int img, int M, int kf, int pa,
+                                        float2 Xa, float2 Xb, float w)
 {
-    kahan_add(acc32, w * fmaf(Xa.x, Xa.x, Xa.y * Xa.y));
-    kahan_add(acc32, w * fmaf(Xb.x, Xb.x, Xb.y * Xb.y));
+    const float2 term = make_float2(w * fmaf(Xa.x, Xa.x, Xa.y * Xa.y),
+                                    w * fmaf(Xb.x, Xb.x, Xb.y * Xb.y));
     if (!o.lp) {
         float *row = o.spec32 + (size_t)(kf - 1) * o.fstride + (size_t)img * 2 * M;
         *reinterpret_cast<float2 *>(row + pa) = make_float2(Xa.x, Xb.x);
         *reinterpret_cast<float2 *>(row + M + pa) = make_float2(Xa.y, Xb.y);
-        return;
+        return term;
     }
     using P = Pair2<T>;
     using V = typename P::V;
@@ -160,15 +166,14 @@ __device__ __forceinline__ void emit2(const SpecOut &o, int img, int M, int kf, 
                       (size_t)img * row_len;
     auto put = [](T *dst, V v) { *reinterpret_cast<V *>(dst) = v; };
     if (!o.split) {
-        kahan_add(acc16, w * fmaf(rf.x, rf.x, imf.x * imf.x));
-        kahan_add(acc16, w * fmaf(rf.y, rf.y, imf.y * imf.y));
         put(r + pa, re2);
         put(r + M + pa, im2);
         if (tmpl) {
             put(r + row_len + pa, __hneg2(im2));  // row 2j+1: [ -im | re | 0 ]
             put(r + row_len + M + pa, re2);
         }
-        return;
+        return make_float2(w * fmaf(rf.x, rf.x, imf.x * imf.x),
+                           w * fmaf(rf.y, rf.y, imf.y * imf.y));
     }
     // FP16 split: lo = x - hi, exact in FP32, rounded to FP16
     const V rel2 = P::pack(Xa.x - rf.x, Xb.x - rf.y);
@@ -184,6 +189,7 @@ __device__ __forceinline__ void emit2(const SpecOut &o, int img, int M, int kf, 
         put(r2 + seg + pa, __hneg2(iml2));
         put(r2 + seg + M + pa, rel2);
     }
+    return term;
 }
 
 __device__ __forceinline__ void cpa16(void *dst, const void *src, int src_bytes)
@@ -236,8 +242,19 @@ __device__ __forceinline__ void stage_levels(const float *__restrict__ qi, int n
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-template <typename T, int nsig>
-__global__ void __launch_bounds__(kSpecThreads, 3)
+// Forms.  The norm of an image is a sum of 256 Kahan sums, one per class c of
+// terms: signal s = c mod nsig of each batch, frequencies k' = c / nsig + (256 /
+// nsig) i in increasing order, batch after batch; every form keeps that order.
+//  - TPC = 1: 256 threads, one per class.
+//  - TPC = 2: 512 threads, where the batch buffers leave room for one CTA per
+//    SM (n > 440): lanes l and l + 16 of a warp take alternate frequencies of
+//    a class and exchange their terms, so both hold the class's sum.
+//  - CL (256 threads): few images; the CTAs of a cluster share an image, CTA r
+//    taking the level batches r, r + S, ...; the terms wait in shared memory,
+//    and after the cluster's barrier CTA 0 adds them in order and finishes the
+//    image.
+template <typename T, int nsig, int TPC, bool CL>
+__global__ void __launch_bounds__(kSpecThreads *TPC, TPC == 2 ? 1 : (CL ? 2 : 3))
 k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2 *__restrict__ tw,
            SpecOut o, float *__restrict__ prof, double *__restrict__ center,
            double *__restrict__ norm32, double *__restrict__ norm16, int parts)
@@ -252,23 +269,42 @@ k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2
     // the next batch's copies while the unpack reads the result
     float2 *bufA = smc;                  // [n nsig]
     float2 *bufB = bufA + n * nsig;      // [n nsig]
-    float2 *x1 = bufB + n * nsig;        // [M] Qhat(1, p) before centring
+    float2 *x1 = bufB + n * nsig;        // [M] Qhat(1, p) before centring (CTA 0's)
     float2 *tws = x1 + M;                // [n] twiddles
-    __shared__ double red[2][kSpecThreads / 32];
+    float2 *terms = tws + n;             // CL: [batches here][NI][256] of levels (pa, pa + 1)
+    constexpr int NW = kSpecThreads * TPC / 32;
+    __shared__ double red[2][NW];
     __shared__ double s_c1[2][2];
     const int Mp = M / parts;  // levels per part
-    const int img = blockIdx.x;
+    int S = 1, rank = 0;
+    if constexpr (CL) {
+        S = (int)cg::this_cluster().num_blocks();
+        rank = (int)cg::this_cluster().block_rank();
+    }
+    const int img = blockIdx.x / S;
     const float *qi = q + (size_t)img * n * M;
-    stage_levels<nsig>(qi, n, M, Mp, parts, 0, bufA);
+    const int nbatch = (M + 2 * nsig - 1) / (2 * nsig);
+    stage_levels<nsig>(qi, n, M, Mp, parts, rank * 2 * nsig, bufA);
     for (int i = threadIdx.x; i < n; i += blockDim.x) tws[i] = tw[i];
+    if constexpr (CL) cg::this_cluster().sync();  // CTA 0 has started: its x1 can be written
+    float2 *x1o = x1;
+    if constexpr (CL) x1o = cg::this_cluster().map_shared_rank(x1, 0);
     const int nh = n / 2;
+    // this thread's class and share of it
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int cls = TPC == 1 ? (int)threadIdx.x : warp * 16 + (lane & 15);
+    const int sub = TPC == 1 ? 0 : lane >> 4;
+    const int s = cls % nsig, a = cls / nsig;
+    constexpr int NA = kSpecThreads / nsig;
+    const int NI = nh / NA + 1;  // frequencies of a class at most
     // norms as compensated (Kahan) FP32 sums: FP64 arithmetic is scarce on
     // this part
-    DF acc32 = {0.f, 0.f}, acc16 = {0.f, 0.f};
+    DF acc = {0.f, 0.f};
     const float invn = 1.f / (float)n;
 
     float2 *cur = bufA, *oth = bufB;
-    for (int p0 = 0; p0 < M; p0 += 2 * nsig) {
+    for (int bt = rank; bt < nbatch; bt += S) {
+        const int p0 = bt * 2 * nsig;
         // ---- batch: levels (p0 + 2s, p0 + 2s + 1) as signal s (re, im)
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncthreads();
@@ -276,43 +312,108 @@ k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2
         // the next batch goes to the buffer the transform did not end in
         // (fft_smem ends with a block barrier: both buffers' readers are done)
         float2 *nxt = R == cur ? oth : cur;
-        if (p0 + 2 * nsig < M) stage_levels<nsig>(qi, n, M, Mp, parts, p0 + 2 * nsig, nxt);
+        if (bt + S < nbatch)
+            stage_levels<nsig>(qi, n, M, Mp, parts, (bt + S) * 2 * nsig, nxt);
         cur = nxt;
         oth = R;
         // ---- unpack two real spectra per signal, k' = 0..n/2
-        for (int t = threadIdx.x; t < (nh + 1) * nsig; t += blockDim.x) {
-            const int kf = t / nsig, s = t % nsig;
-            const float2 Z = R[kf * nsig + s];
-            const float2 Zc = cconj(R[(kf ? n - kf : 0) * nsig + s]);
-            // Xa = (Z + conj Z(n-k))/2, Xb = (Z - conj Z(n-k)) / (2i)
-            const float2 Xa = make_float2(0.5f * (Z.x + Zc.x), 0.5f * (Z.y + Zc.y));
-            const float2 dz = make_float2(0.5f * (Z.x - Zc.x), 0.5f * (Z.y - Zc.y));
-            const float2 Xb = make_float2(dz.y, -dz.x);
-            const int pa = p0 + 2 * s, pb = pa + 1;
-            if (kf >= 2 && (M & 1) == 0 && pb < M) {
-                // both levels at once (pa even, M even: 4-byte aligned pairs)
-                float2 A = Xa, Bv = Xb;
-                if (kf == nh) A.y = Bv.y = 0.f;  // Nyquist term of a real signal
-                emit2<T>(o, img, M, kf, pa, A, Bv, kf == nh ? 1.f : 2.f, acc32, acc16);
-                continue;
-            }
-#pragma unroll
-            for (int h2 = 0; h2 < 2; ++h2) {
-                const int p = h2 ? pb : pa;
-                if (p >= M) continue;
-                float2 X = h2 ? Xb : Xa;
-                if (kf == 0) {
-                    prof[(size_t)img * M + p] = X.x * invn;
-                } else if (kf == 1) {
-                    x1[p] = X;
-                } else {
-                    if (kf == nh) X.y = 0.f;  // Nyquist term of a real signal
+        const int pa = p0 + 2 * s, pb = pa + 1;
+        for (int i0 = 0; i0 < NI; i0 += TPC) {
+            const int i = i0 + sub, kf = a + NA * i;
+            float2 term = make_float2(0.f, 0.f);
+            if (kf <= nh) {
+                const float2 Z = R[kf * nsig + s];
+                const float2 Zc = cconj(R[(kf ? n - kf : 0) * nsig + s]);
+                // Xa = (Z + conj Z(n-k))/2, Xb = (Z - conj Z(n-k)) / (2i)
+                float2 Xa = make_float2(0.5f * (Z.x + Zc.x), 0.5f * (Z.y + Zc.y));
+                const float2 dz = make_float2(0.5f * (Z.x - Zc.x), 0.5f * (Z.y - Zc.y));
+                float2 Xb = make_float2(dz.y, -dz.x);
+                if (kf >= 2) {
+                    if (kf == nh) Xa.y = Xb.y = 0.f;  // Nyquist term of a real signal
                     const float w = kf == nh ? 1.f : 2.f;
-                    emit<T>(o, img, M, kf, p, X, w, acc32, acc16);
+                    if ((M & 1) == 0) {
+                        // both levels at once (pa even, M even: 4-byte aligned pairs)
+                        if (pb < M) {
+                            term = emit2<T>(o, img, M, kf, pa, Xa, Xb, w);
+                            if constexpr (!CL && TPC == 1) {
+                                kahan_add(acc, term.x);
+                                kahan_add(acc, term.y);
+                            }
+                        }
+                    } else {
+                        if (pa < M) {
+                            term.x = emit<T>(o, img, M, kf, pa, Xa, w);
+                            if constexpr (!CL && TPC == 1) kahan_add(acc, term.x);
+                        }
+                        if (pb < M) {
+                            term.y = emit<T>(o, img, M, kf, pb, Xb, w);
+                            if constexpr (!CL && TPC == 1) kahan_add(acc, term.y);
+                        }
+                    }
+                } else if (kf == 1) {
+                    if (pa < M) x1o[pa] = Xa;
+                    if (pb < M) x1o[pb] = Xb;
+                } else {
+                    if (pa < M) prof[(size_t)img * M + pa] = Xa.x * invn;
+                    if (pb < M) prof[(size_t)img * M + pb] = Xb.x * invn;
+                }
+            }
+            if constexpr (CL) {
+                terms[((bt / S) * NI + i) * kSpecThreads + cls] = term;
+            } else if constexpr (TPC == 2) {
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const float2 tu =
+                        make_float2(__shfl_sync(0xffffffffu, term.x, (lane & 15) + 16 * u),
+                                    __shfl_sync(0xffffffffu, term.y, (lane & 15) + 16 * u));
+                    const int ku = a + NA * (i0 + u);
+                    if (ku >= 2 && ku <= nh) {
+                        if (pa < M) kahan_add(acc, tu.x);
+                        if (pb < M) kahan_add(acc, tu.y);
+                    }
                 }
             }
         }
         __syncthreads();
+    }
+    const bool tmpl = img >= o.Nq;
+    // ---- zero padding of the low-precision rows: [2M, ldk) of every segment
+    if (o.lp && o.ldk > 2 * M) {
+        const int pad = o.ldk - 2 * M;
+        const int nseg = o.split ? 2 : 1;
+        const int row_len = nseg * o.ldk;
+        const int rows = tmpl ? 2 : 1;
+        const int per_f = rows * nseg * pad;
+        for (int t = rank * blockDim.x + threadIdx.x; t < nh * per_f; t += S * blockDim.x) {
+            const int kf = 1 + t / per_f, rem = t % per_f;
+            const int rr = rem / (nseg * pad), sg = (rem / pad) % nseg, e = 2 * M + rem % pad;
+            T *r = tmpl ? reinterpret_cast<T *>(o.lp_t) + (size_t)(kf - 1) * o.lpt_fstride +
+                              (size_t)(2 * (img - o.Nq) + rr) * row_len
+                        : reinterpret_cast<T *>(o.lp_q) + (size_t)(kf - 1) * o.lpq_fstride +
+                              (size_t)img * row_len;
+            r[sg * o.ldk + e] = to_lp<T>(0.f);
+        }
+    }
+    if constexpr (CL) {
+        cg::this_cluster().sync();  // every batch's terms and x1 are in place
+        if (rank == 0) {
+            for (int bt = 0; bt < nbatch; ++bt) {
+                const int pa = bt * 2 * nsig + 2 * s, pb = pa + 1;
+                const float2 *tr = cg::this_cluster().map_shared_rank(terms, bt % S) +
+                                   (size_t)(bt / S) * NI * kSpecThreads + cls;
+#pragma unroll 8
+                for (int i = 0; i < NI; ++i) {
+                    const int ku = a + NA * i;
+                    const float2 tu = tr[i * kSpecThreads];
+                    if (ku >= 2 && ku <= nh) {
+                        if (pa < M) kahan_add(acc, tu.x);
+                        if (pb < M) kahan_add(acc, tu.y);
+                    }
+                }
+            }
+        }
+        cg::this_cluster().sync();  // CTA 0 has read the other CTAs' terms
+        if (rank != 0) return;
     }
     // ---- centring, per part: c1 = mean_p Qhat_u(1, p);  a = (2/n)(Re c1, -Im c1)
     for (int part = 0; part < parts; ++part) {
@@ -321,7 +422,6 @@ k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2
             cr += x1[p].x;
             ci += x1[p].y;
         }
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
         for (int off = 16; off; off >>= 1) {
             cr += __shfl_xor_sync(0xffffffffu, cr, off);
@@ -334,7 +434,7 @@ k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2
         __syncthreads();
         if (threadIdx.x == 0) {
             double sr = 0.0, si = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+            for (int w = 0; w < NW; ++w) {
                 sr += red[0][w];
                 si += red[1][w];
             }
@@ -346,53 +446,26 @@ k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2
         }
         __syncthreads();
     }
-    for (int p = threadIdx.x; p < M; p += blockDim.x) {
-        const int part = p / Mp;
-        const float c1r = (float)s_c1[part][0], c1i = (float)s_c1[part][1];
-        const float2 X = make_float2(x1[p].x - c1r, x1[p].y - c1i);
-        emit<T>(o, img, M, 1, p, X, 2.f, acc32, acc16);  // n >= 4: k' = 1 < n/2
-    }
-    // ---- zero padding of the low-precision rows: [2M, ldk) of every segment
-    if (o.lp && o.ldk > 2 * M) {
-        const int pad = o.ldk - 2 * M;
-        const bool tmpl = img >= o.Nq;
-        const int nseg = o.split ? 2 : 1;
-        const int row_len = nseg * o.ldk;
-        const int rows = tmpl ? 2 : 1;
-        const int per_f = rows * nseg * pad;
-        for (int t = threadIdx.x; t < nh * per_f; t += blockDim.x) {
-            const int kf = 1 + t / per_f, rem = t % per_f;
-            const int rr = rem / (nseg * pad), sg = (rem / pad) % nseg, e = 2 * M + rem % pad;
-            T *r = tmpl ? reinterpret_cast<T *>(o.lp_t) + (size_t)(kf - 1) * o.lpt_fstride +
-                              (size_t)(2 * (img - o.Nq) + rr) * row_len
-                        : reinterpret_cast<T *>(o.lp_q) + (size_t)(kf - 1) * o.lpq_fstride +
-                              (size_t)img * row_len;
-            r[sg * o.ldk + e] = to_lp<T>(0.f);
+    // k' = 1 (n >= 4: 1 < n/2), last in each class: level p is class p mod 256's
+    if (sub == 0) {
+        for (int p = cls; p < M; p += kSpecThreads) {
+            const int part = p / Mp;
+            const float c1r = (float)s_c1[part][0], c1i = (float)s_c1[part][1];
+            const float2 X = make_float2(x1[p].x - c1r, x1[p].y - c1i);
+            kahan_add(acc, emit<T>(o, img, M, 1, p, X, 2.f));
         }
     }
     // ---- norms: Parseval over k' != 0 of the centred spectra, / n
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double a32 = (double)acc32.hi + (double)acc32.lo;
-    double a16 = (double)acc16.hi + (double)acc16.lo;
+    double an = sub == 0 ? (double)acc.hi + (double)acc.lo : 0.0;
 #pragma unroll
-    for (int off = 16; off; off >>= 1) {
-        a32 += __shfl_xor_sync(0xffffffffu, a32, off);
-        a16 += __shfl_xor_sync(0xffffffffu, a16, off);
-    }
+    for (int off = 16; off; off >>= 1) an += __shfl_xor_sync(0xffffffffu, an, off);
     __syncthreads();
-    if (lane == 0) {
-        red[0][warp] = a32;
-        red[1][warp] = a16;
-    }
+    if (lane == 0) red[0][warp] = an;
     __syncthreads();
     if (threadIdx.x == 0) {
-        double s32 = 0.0, s16 = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            s32 += red[0][w];
-            s16 += red[1][w];
-        }
-        norm32[img] = s32 / n;
-        if (norm16) norm16[img] = s16 / n;
+        double sn = 0.0;
+        for (int w = 0; w < NW; ++w) sn += red[0][w];
+        (o.lp && !o.split ? norm16 : norm32)[img] = sn / n;
     }
 }
 
@@ -419,24 +492,62 @@ cudaError_t launch_spectrum(const float *q, int nb, int n, int M, const FftPlan 
     if (smem > kSmemOptIn) return cudaErrorInvalidValue;
     SpecOut o{spec32, fstride, lp_q, lpq_fstride, lp_t, lpt_fstride, Nq, tc_ldk(M),
               lp_kind != 0, lp_kind == 3};
-#define SW_SPEC_LAUNCH(T, NS)                                                                    \
-    do {                                                                                        \
-        cudaFuncSetAttribute(k_spectrum<T, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
-                             (int)smem);                                                        \
-        k_spectrum<T, NS><<<nb, kSpecThreads, smem, st>>>(q, n, M, plan, tw, o, prof, center,  \
-                                                          norm32, norm16, parts);               \
-    } while (0)
-    if (lp_kind == 2 || lp_kind == 3) {
-        if (nsig == 16) SW_SPEC_LAUNCH(__half, 16);
-        else if (nsig == 8) SW_SPEC_LAUNCH(__half, 8);
-        else SW_SPEC_LAUNCH(__half, 4);
-    } else {
-        if (nsig == 16) SW_SPEC_LAUNCH(__nv_bfloat16, 16);
-        else if (nsig == 8) SW_SPEC_LAUNCH(__nv_bfloat16, 8);
-        else SW_SPEC_LAUNCH(__nv_bfloat16, 4);
+    // form: a cluster per image while all images' CTAs are resident at once;
+    // else 512 threads where an SM holds one CTA
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const int nbatch = (M + 2 * nsig - 1) / (2 * nsig);
+    const size_t per_batch = sizeof(float2) * (size_t)((n / 2) / (kSpecThreads / nsig) + 1) *
+                             kSpecThreads;
+    int S = 1;
+    size_t smem_cl = smem;
+    for (int w = std::min(8, nbatch); w > 1; --w) {
+        const size_t need = smem + per_batch * ((nbatch + w - 1) / w);
+        const int per_sm = need <= kSmemOptIn / 2 ? 2 : 1;
+        // (a cluster stays within one of the at least eight GPCs)
+        // (a narrow cluster loses its gain to the two barriers and the ordered
+        // sum: 80 images of four batches take 28 us on clusters of 3 or alone)
+        if (nbatch - (nbatch + w - 1) / w < 3) break;
+        if (need <= kSmemOptIn && nb <= 8 * (sms / 8 * per_sm / w)) {
+            S = w;
+            smem_cl = need;
+            break;
+        }
     }
-#undef SW_SPEC_LAUNCH
-    return cudaGetLastError();
+    auto run = [&](auto kern, int threads, int width, size_t bytes) {
+        cudaError_t er = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)bytes);
+        if (er != cudaSuccess) return er;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(nb * width));
+        cfg.blockDim = dim3((unsigned)threads);
+        cfg.dynamicSmemBytes = bytes;
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)width;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = width > 1 ? 1 : 0;
+        return cudaLaunchKernelEx(&cfg, kern, q, n, M, plan, tw, o, prof, center, norm32, norm16,
+                                  parts);
+    };
+    const bool wide = smem > kSmemOptIn / 2;
+#define SW_SPEC_FORMS(T, NS)                                                               \
+    return S > 1    ? run(k_spectrum<T, NS, 1, true>, kSpecThreads, S, smem_cl)            \
+           : wide   ? run(k_spectrum<T, NS, 2, false>, 2 * kSpecThreads, 1, smem)          \
+                    : run(k_spectrum<T, NS, 1, false>, kSpecThreads, 1, smem)
+    if (lp_kind == 2 || lp_kind == 3) {
+        if (nsig == 16) SW_SPEC_FORMS(__half, 16);
+        if (nsig == 8) SW_SPEC_FORMS(__half, 8);
+        SW_SPEC_FORMS(__half, 4);
+    }
+    if (nsig == 16) SW_SPEC_FORMS(__nv_bfloat16, 16);
+    if (nsig == 8) SW_SPEC_FORMS(__nv_bfloat16, 8);
+    SW_SPEC_FORMS(__nv_bfloat16, 4);
+#undef SW_SPEC_FORMS
 }
 
 }  // namespace swk
