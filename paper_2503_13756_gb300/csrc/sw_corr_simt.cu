@@ -11,6 +11,8 @@
 // 16 at a time in shared memory (transposed so that each thread reads four
 // consecutive queries or templates as one float4), register double-buffer
 // of the next stage.
+#include <algorithm>
+
 #include "sw_internal.cuh"
 
 namespace swk {
@@ -95,12 +97,57 @@ k_corr_simt(const float *__restrict__ X, size_t xf, const float *__restrict__ Y,
     }
 }
 
+// A few pairs (a single pair above all): one thread per frequency and pair, in
+// the tile kernel's order of operations.  Where the 64 x 64 tile is nearly
+// all padding its time is the latency of its stages (a pair at n = 360, M =
+// 128: 31 us); here a CTA copies the rows of `fb` frequencies to shared memory
+// at once and each thread runs one chain of 2 M dependent FMAs per component
+// (4 us).  Rows are 2 M floats; a frequency's rows take an odd number of
+// floats, so that the threads of adjacent frequencies read distinct banks.
+__global__ void __launch_bounds__(256)
+k_corr_few(const float *__restrict__ X, size_t xf, const float *__restrict__ Y, size_t yf, int Nq,
+           int Nt, int M, int nf, int fb, float2 *__restrict__ C)
+{
+    extern __shared__ float sm[];
+    const int M2 = 2 * M, rows = Nq + Nt, FS = rows * M2 + 1;
+    const int f0 = blockIdx.x * fb, nb = min(fb, nf - f0);
+    for (int fl = 0; fl < nb; ++fl) {
+        const float *Xf = X + (size_t)(f0 + fl) * xf, *Yf = Y + (size_t)(f0 + fl) * yf;
+#pragma unroll 4
+        for (int e = threadIdx.x; e < rows * M2; e += blockDim.x)
+            sm[fl * FS + e] = e < Nq * M2 ? __ldg(Xf + e) : __ldg(Yf + e - Nq * M2);
+    }
+    __syncthreads();
+    const int pairs = Nq * Nt;
+    for (int t = threadIdx.x; t < nb * pairs; t += blockDim.x) {
+        const int fl = t / pairs, pr = t % pairs, i = pr / Nt, j = pr % Nt;
+        const float *x = sm + fl * FS + i * M2, *y = sm + fl * FS + (Nq + j) * M2;
+        float re = 0.f, im = 0.f;
+#pragma unroll 8
+        for (int p = 0; p < M; ++p) {
+            const float a = x[p], b = x[M + p], c = y[p], d = y[M + p];
+            re = fmaf(a, c, fmaf(b, d, re));
+            im = fmaf(b, c, fmaf(-a, d, im));
+        }
+        C[((size_t)(f0 + fl) * Nq + i) * Nt + j] = make_float2(re, im);
+    }
+}
+
 }  // namespace
 
 cudaError_t launch_corr_simt(const float *X, size_t xf, const float *Y, size_t yf, int Nq,
                              int Nt, int M, int nf, float2 *C, cudaStream_t st)
 {
     if (Nq <= 0 || Nt <= 0 || nf <= 0) return cudaSuccess;
+    // few pairs: frequencies per CTA so that its rows fit 48 KB and the chip
+    // has a CTA or two per SM (see k_corr_few)
+    const size_t per_f = sizeof(float) * ((size_t)(Nq + Nt) * 2 * M + 1);
+    if (Nq <= 16 && Nt <= 16 && Nq * Nt <= 64 && per_f <= 48 * 1024) {
+        const int fb = (int)std::max<size_t>(
+            1, std::min<size_t>({48 * 1024 / per_f, (size_t)(nf + 151) / 152, (size_t)8}));
+        k_corr_few<<<(nf + fb - 1) / fb, 256, per_f * fb, st>>>(X, xf, Y, yf, Nq, Nt, M, nf, fb, C);
+        return cudaGetLastError();
+    }
     dim3 grid((Nt + TN - 1) / TN, (Nq + TM - 1) / TM, nf);
     k_corr_simt<<<grid, 256, 0, st>>>(X, xf, Y, yf, Nq, Nt, M, C);
     return cudaGetLastError();

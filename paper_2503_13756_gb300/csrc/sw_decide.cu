@@ -724,22 +724,31 @@ k_decide_reg(DecideArgs A, const float2 *__restrict__ tw)
         res_d[2 * s + lane] = lane ? db : da;
     }
     double aix, aiy, dix, diy;
-    // ---- full curve of pair (0, 0) (single-pair call)
-    if (A.curve && i == 0 && j0 == 0 && s == 0) {
-        centre_of(A.ctr_q, i, PARTS, aix, aiy, dix, diy);
-        double ajx, ajy, djx, djy;
-        centre_of(A.ctr_t, 0, PARTS, ajx, ajy, djx, djy);
-        const double base = (double)da + A.norm_q[0] + A.norm_t[0];
-        const int st = A.st_q[0] || stt[0] || (A.dev_err && *A.dev_err);
-        if (live) {
+    // full curve of pair (0, 0) (single-pair call): its values, through the
+    // twiddles' place once every warp has read those
+    const bool curve = A.curve && i == 0 && j0 == 0;
+    float *cv = reinterpret_cast<float *>(tws);
+    if (curve) {
+        __syncthreads();
+        if (s == 0 && live) {
 #pragma unroll
-            for (int k1 = 0; k1 < MW; ++k1)
-                curve_point<PARTS>(A, k1 + lb, v[k1].x, base, st, X.tmode, aix, aiy, dix, diy,
-                                   ajx, ajy, djx, djy);
+            for (int k1 = 0; k1 < MW; ++k1) cv[k1 + lb] = v[k1].x;
         }
     }
     // every warp has posted its pairs
     __syncthreads();
+    // ---- the curve, FP64: its points over all threads (in the one warp that
+    // holds the values, twelve points a lane in series took 5 us at n = 360)
+    if (curve) {
+        centre_of(A.ctr_q, 0, PARTS, aix, aiy, dix, diy);
+        double ajx, ajy, djx, djy;
+        centre_of(A.ctr_t, 0, PARTS, ajx, ajy, djx, djy);
+        const double base = (double)res_d[0] + A.norm_q[0] + A.norm_t[0];
+        const int st = A.st_q[0] || stt[0] || (A.dev_err && *A.dev_err);
+        for (int l = tid; l < n; l += kRegThreads)
+            curve_point<PARTS>(A, l, cv[l], base, st, X.tmode, aix, aiy, dix, diy, ajx, ajy, djx,
+                               djy);
+    }
     // ---- FP64 distance at l*: one lane per template, all in warp 0 (the
     // FP64 pipe is narrow: its instructions are issued once per 16 pairs)
     if (warp == 0 && lane < kRegTemplates && j0 + lane < Nt) {
