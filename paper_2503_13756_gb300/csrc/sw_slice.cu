@@ -190,8 +190,8 @@ __device__ __forceinline__ void slice_grid(const SliceArgs &A, const float *__re
     const int nleft = slice_left(N), nright = slice_right(N);
     // ---- A: one warp per column pair (c, c+1): FFT along r', kept rows.
     // fetch(r) gives the pixels (r, c) and (r, c + 1).
-    auto column_pair = [&](int c, auto fetch) {
-        float2 v[M];
+    auto read_pair = [&](float2 (&v)[M], int c, auto fetch) {
+        if (c >= L) return;
         const float pc0 = __ldg(A.psi_inv + c), pc1 = c + 1 < L ? __ldg(A.psi_inv + c + 1) : 0.f;
 #pragma unroll
         for (int n1 = 0; n1 < M; ++n1) {
@@ -215,6 +215,9 @@ __device__ __forceinline__ void slice_grid(const SliceArgs &A, const float *__re
                 v[n1] = make_float2(x.x * pc0 * pr, x.y * pc1 * pr);
             }
         }
+    };
+    auto transform_pair = [&](float2 (&v)[M], int c) {
+        if (c >= L) return;
         warp_ifft<M>(v, tw, lane);
         // Z[kout] = v[k1], kout = k1 + M brev5(lane); Z[-kout] sits on lane
         // brev5(32 - brev5(lane)) slot 0 (k1 = 0), else lane 31 - lane slot M - k1
@@ -236,8 +239,96 @@ __device__ __forceinline__ void slice_grid(const SliceArgs &A, const float *__re
             }
         }
     };
+    auto column_pair = [&](int c, auto fetch) {
+        float2 v[M];
+        read_pair(v, c, fetch);
+        transform_pair(v, c);
+    };
+    // ---- B: one warp per kept row: FFT along c', left and right columns
+    auto rows_phase = [&] {
+        for (int i = rank + P * warp; i < rows; i += P * nw) {
+            float2 v[M];
+#pragma unroll
+            for (int n1 = 0; n1 < M; ++n1) {
+                const int n = 32 * n1 + lane;
+                const int c = (n < N / 2 ? n : n - N) + half;
+                v[n1] = (c >= 0 && c < L) ? G[i * S + c] : make_float2(0.f, 0.f);
+            }
+            __syncwarp();
+            warp_ifft<M>(v, tw, lane);
+            const int kb = M * brev5(lane);
+#pragma unroll
+            for (int k1 = 0; k1 < M; ++k1) {
+                const int kout = k1 + kb;
+                const int q = wrap_n(kout - lo, N);  // left column with l1 = kout (mod N)
+                if (q < nleft) G[i * S + q] = v[k1];
+                if (kout >= 1 && kout <= nright) G[i * S + nleft + nright - kout] = v[k1];
+            }
+            if constexpr (CL && SHARED) {  // the finished row to the other CTAs, coalesced
+                __syncwarp();
+                for (int r = 1; r < P; ++r) {
+                    float2 *Gr = cg::this_cluster().map_shared_rank(G, (rank + r) & (P - 1));
+                    for (int x = lane; x < nleft + nright; x += 32) Gr[i * S + x] = G[i * S + x];
+                }
+            }
+        }
+    };
+    if constexpr (SHARED && !CL) {
+        if (A.srcL == L) {
+            // The image through the (idle) sample buffer in bands of one column
+            // pair per warp: coalesced loads, both bands in flight at once, and
+            // the second band's copy beside the first band's transforms.  Read
+            // straight from global memory, each lane takes 8 bytes of another
+            // row, one sector request per lane (0.418 against 0.408 us per
+            // 128 x 128 image at n = 256, 0.206 against 0.199 at L = 64).
+            constexpr int NWC = kSliceThreads / 32, BW = 2 * NWC, RSB = BW + 1;
+            constexpr int PER = (128 * BW) / kSliceThreads;  // values per thread and band
+            static_assert(kSliceThreads % BW == 0, "a thread keeps its column of the band");
+            const int cc = threadIdx.x % BW, r0 = threadIdx.x / BW;
+            constexpr int RSTEP = kSliceThreads / BW;
+            float x0[PER], x1[PER];
+            auto load = [&](float (&x)[PER], int cb) {
+#pragma unroll
+                for (int u = 0; u < PER; ++u) {
+                    const int r = r0 + u * RSTEP;
+                    x[u] = r < L && cb + cc < L ? __ldg(src + (size_t)r * L + cb + cc) : 0.f;
+                }
+            };
+            auto store = [&](const float (&x)[PER]) {
+#pragma unroll
+                for (int u = 0; u < PER; ++u) {
+                    const int r = r0 + u * RSTEP;
+                    if (r < L) stage[r * RSB + cc] = x[u];
+                }
+            };
+            auto fetch = [&](int r) {
+                const float *row = stage + r * RSB + 2 * warp;
+                return make_float2(row[0], row[1]);
+            };
+            load(x0, 0);
+            const bool two = L > BW;
+            if (two) load(x1, BW);
+            store(x0);
+            __syncthreads();
+            float2 v[M];
+            read_pair(v, 2 * warp, fetch);
+            if (two) {
+                __syncthreads();
+                store(x1);
+            }
+            transform_pair(v, 2 * warp);
+            if (two) {
+                __syncthreads();
+                read_pair(v, BW + 2 * warp, fetch);
+                transform_pair(v, BW + 2 * warp);
+            }
+            __syncthreads();
+            rows_phase();
+            return;
+        }
+    }
     constexpr int BW = 32, RSB = BW + 1;  // band width; staged row stride (odd: rows on distinct banks)
-    if (stage != nullptr && A.srcL == L && 2 * nw == BW) {
+    if (!SHARED && stage != nullptr && A.srcL == L && 2 * nw == BW) {
         const int nbands = (L + BW - 1) / BW;
         auto issue = [&](int b, float *buf) {
             const int cb = b * BW, w = min(BW, L - cb);
@@ -289,33 +380,7 @@ __device__ __forceinline__ void slice_grid(const SliceArgs &A, const float *__re
             });
     }
     image_sync<CL>();
-    // ---- B: one warp per kept row: FFT along c', left and right columns
-    for (int i = rank + P * warp; i < rows; i += P * nw) {
-        float2 v[M];
-#pragma unroll
-        for (int n1 = 0; n1 < M; ++n1) {
-            const int n = 32 * n1 + lane;
-            const int c = (n < N / 2 ? n : n - N) + half;
-            v[n1] = (c >= 0 && c < L) ? G[i * S + c] : make_float2(0.f, 0.f);
-        }
-        __syncwarp();
-        warp_ifft<M>(v, tw, lane);
-        const int kb = M * brev5(lane);
-#pragma unroll
-        for (int k1 = 0; k1 < M; ++k1) {
-            const int kout = k1 + kb;
-            const int q = wrap_n(kout - lo, N);  // left column with l1 = kout (mod N)
-            if (q < nleft) G[i * S + q] = v[k1];
-            if (kout >= 1 && kout <= nright) G[i * S + nleft + nright - kout] = v[k1];
-        }
-        if constexpr (CL && SHARED) {  // the finished row to the other CTAs, coalesced
-            __syncwarp();
-            for (int r = 1; r < P; ++r) {
-                float2 *Gr = cg::this_cluster().map_shared_rank(G, (rank + r) & (P - 1));
-                for (int x = lane; x < nleft + nright; x += 32) Gr[i * S + x] = G[i * S + x];
-            }
-        }
-    }
+    rows_phase();
 }
 
 // Tap weights along each axis from the target's offsets (x1, x2) from its
@@ -716,7 +781,8 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_project_slice(SliceArgs A)
     for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = A.tw[i];
     image_sync<CL>();
     int bad = 0, mass = 0;
-    slice_grid<M, CL>(A, image_of(A, gi), G, tw, warp, kSliceThreads / 32, lane, bad, mass);
+    slice_grid<M, CL>(A, image_of(A, gi), G, tw, warp, kSliceThreads / 32, lane, bad, mass,
+                      reinterpret_cast<float *>(Xs));
     image_status<CL>(A, gi, &s_flags, bad, mass);
     const int step = kSliceBatch * (CL ? (int)cg::this_cluster().num_blocks() : 1);
     for (int k0 = 0; k0 < A.nh; k0 += step) {
@@ -751,7 +817,8 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_project_slice_up(SliceArgs
     for (int i = threadIdx.x; i < 2 * N; i += blockDim.x) tw2[i] = A.tw2[i];
     image_sync<CL>();
     int bad = 0, mass = 0;
-    slice_grid<MG, CL>(A, image_of(A, gi), G, tw, warp, kSliceThreads / 32, lane, bad, mass);
+    slice_grid<MG, CL>(A, image_of(A, gi), G, tw, warp, kSliceThreads / 32, lane, bad, mass,
+                       reinterpret_cast<float *>(Xs));
     image_status<CL>(A, gi, &s_flags, bad, mass);
     const int step = kUpBatch * (CL ? (int)cg::this_cluster().num_blocks() : 1);
     for (int k0 = 0; k0 < A.nh; k0 += step) {
