@@ -243,22 +243,30 @@ __device__ __forceinline__ void stage_levels(const float *__restrict__ qi, int n
 }
 
 // Forms.  The norm of an image is a sum of 256 Kahan sums, one per class c of
-// terms: signal s = c mod nsig of each batch, frequencies k' = c / nsig + (256 /
-// nsig) i in increasing order, batch after batch; every form keeps that order.
-//  - TPC = 1: 256 threads, one per class.
-//  - TPC = 2: 512 threads, where the batch buffers leave room for one CTA per
-//    SM (n > 440): lanes l and l + 16 of a warp take alternate frequencies of
-//    a class and exchange their terms, so both hold the class's sum.
-//  - CL (256 threads): few images; the CTAs of a cluster share an image, CTA r
-//    taking the level batches r, r + S, ...; the terms wait in shared memory,
-//    and after the cluster's barrier CTA 0 adds them in order and finishes the
-//    image.
-template <typename T, int nsig, int TPC, bool CL>
-__global__ void __launch_bounds__(kSpecThreads *TPC, TPC == 2 ? 1 : (CL ? 2 : 3))
+// terms: with NSC signals to a batch, signal c mod NSC of each batch at the
+// frequencies k' = c / NSC + (256 / NSC) i in increasing order, batch after
+// batch; every form keeps that order.
+//  - plain: batches of NSC signals, one thread per class.
+//  - HB, where the plain form's buffers leave room for fewer than three CTAs
+//    per SM (n > 256 at NSC = 16): half batches of NSC / 2 signals, so half of
+//    the buffers and more CTAs on an SM.  Lanes l and l + 16 of a warp take
+//    alternate frequencies of a class and exchange their terms, so both hold
+//    its sum, and a thread keeps two classes, one per half of the batch.
+//    10,001 images at n = 512, M = 256: 5.2 ms plain (one CTA of 8 warps per
+//    SM), 4.9 ms with 512 threads on full batches, 3.9 ms in this form.  Not
+//    for images that the plain form holds all at once: their time is that of
+//    one image's batches in turn (128 images at n = 360, M = 256: 68 us plain,
+//    90 us in this form).
+//  - CL: few images; the CTAs of a cluster share an image, CTA r taking the
+//    level batches r, r + S, ...; the terms wait in shared memory, and after
+//    the cluster's barrier CTA 0 adds them in order and finishes the image.
+template <typename T, int NSC, bool HB, bool CL>
+__global__ void __launch_bounds__(kSpecThreads, CL ? 2 : 3)
 k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2 *__restrict__ tw,
            SpecOut o, float *__restrict__ prof, double *__restrict__ center,
            double *__restrict__ norm32, double *__restrict__ norm16, int parts)
 {
+    constexpr int nsig = HB ? NSC / 2 : NSC;  // signals transformed at a time
     // M levels in all; with parts = 2 (ramp-filtered distance) the levels
     // [0, M/2) and [M/2, M) are the quantiles of the positive and negative
     // parts, stored as [parts][n][M/2], and each part is centred by its own
@@ -272,7 +280,7 @@ k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2
     float2 *x1 = bufB + n * nsig;        // [M] Qhat(1, p) before centring (CTA 0's)
     float2 *tws = x1 + M;                // [n] twiddles
     float2 *terms = tws + n;             // CL: [batches here][NI][256] of levels (pa, pa + 1)
-    constexpr int NW = kSpecThreads * TPC / 32;
+    constexpr int NW = kSpecThreads / 32;
     __shared__ double red[2][NW];
     __shared__ double s_c1[2][2];
     const int Mp = M / parts;  // levels per part
@@ -290,16 +298,16 @@ k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2
     float2 *x1o = x1;
     if constexpr (CL) x1o = cg::this_cluster().map_shared_rank(x1, 0);
     const int nh = n / 2;
-    // this thread's class and share of it
+    // this thread's class (HB: the first of two) and share of it
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int cls = TPC == 1 ? (int)threadIdx.x : warp * 16 + (lane & 15);
-    const int sub = TPC == 1 ? 0 : lane >> 4;
+    const int cls = HB ? warp * 16 + (lane & 15) : (int)threadIdx.x;
+    const int sub = HB ? lane >> 4 : 0;
     const int s = cls % nsig, a = cls / nsig;
-    constexpr int NA = kSpecThreads / nsig;
+    constexpr int NA = kSpecThreads / NSC;
     const int NI = nh / NA + 1;  // frequencies of a class at most
     // norms as compensated (Kahan) FP32 sums: FP64 arithmetic is scarce on
     // this part
-    DF acc = {0.f, 0.f};
+    DF acc = {0.f, 0.f}, acc_other = {0.f, 0.f};  // HB: this half's and the other half's class
     const float invn = 1.f / (float)n;
 
     float2 *cur = bufA, *oth = bufB;
@@ -318,7 +326,7 @@ k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2
         oth = R;
         // ---- unpack two real spectra per signal, k' = 0..n/2
         const int pa = p0 + 2 * s, pb = pa + 1;
-        for (int i0 = 0; i0 < NI; i0 += TPC) {
+        for (int i0 = 0; i0 < NI; i0 += HB ? 2 : 1) {
             const int i = i0 + sub, kf = a + NA * i;
             float2 term = make_float2(0.f, 0.f);
             if (kf <= nh) {
@@ -335,7 +343,7 @@ k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2
                         // both levels at once (pa even, M even: 4-byte aligned pairs)
                         if (pb < M) {
                             term = emit2<T>(o, img, M, kf, pa, Xa, Xb, w);
-                            if constexpr (!CL && TPC == 1) {
+                            if constexpr (!CL && !HB) {
                                 kahan_add(acc, term.x);
                                 kahan_add(acc, term.y);
                             }
@@ -343,11 +351,11 @@ k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2
                     } else {
                         if (pa < M) {
                             term.x = emit<T>(o, img, M, kf, pa, Xa, w);
-                            if constexpr (!CL && TPC == 1) kahan_add(acc, term.x);
+                            if constexpr (!CL && !HB) kahan_add(acc, term.x);
                         }
                         if (pb < M) {
                             term.y = emit<T>(o, img, M, kf, pb, Xb, w);
-                            if constexpr (!CL && TPC == 1) kahan_add(acc, term.y);
+                            if constexpr (!CL && !HB) kahan_add(acc, term.y);
                         }
                     }
                 } else if (kf == 1) {
@@ -360,7 +368,7 @@ k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2
             }
             if constexpr (CL) {
                 terms[((bt / S) * NI + i) * kSpecThreads + cls] = term;
-            } else if constexpr (TPC == 2) {
+            } else if constexpr (HB) {
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
                     const float2 tu =
@@ -374,7 +382,19 @@ k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2
                 }
             }
         }
+        if constexpr (HB) {  // the next half batch adds to the other class
+            const DF t = acc;
+            acc = acc_other;
+            acc_other = t;
+        }
         __syncthreads();
+    }
+    if constexpr (HB) {
+        if (nbatch & 1) {  // acc: the first half's class again
+            const DF t = acc;
+            acc = acc_other;
+            acc_other = t;
+        }
     }
     const bool tmpl = img >= o.Nq;
     // ---- zero padding of the low-precision rows: [2M, ldk) of every segment
@@ -447,16 +467,22 @@ k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2
         __syncthreads();
     }
     // k' = 1 (n >= 4: 1 < n/2), last in each class: level p is class p mod 256's
-    if (sub == 0) {
-        for (int p = cls; p < M; p += kSpecThreads) {
+    auto first_frequency = [&](int c, DF &sum) {
+        for (int p = c; p < M; p += kSpecThreads) {
             const int part = p / Mp;
             const float c1r = (float)s_c1[part][0], c1i = (float)s_c1[part][1];
             const float2 X = make_float2(x1[p].x - c1r, x1[p].y - c1i);
-            kahan_add(acc, emit<T>(o, img, M, 1, p, X, 2.f));
+            kahan_add(sum, emit<T>(o, img, M, 1, p, X, 2.f));
         }
+    };
+    if (sub == 0) {
+        first_frequency(a * NSC + s, acc);
+        if constexpr (HB) first_frequency(a * NSC + s + nsig, acc_other);
     }
     // ---- norms: Parseval over k' != 0 of the centred spectra, / n
-    double an = sub == 0 ? (double)acc.hi + (double)acc.lo : 0.0;
+    double an = (double)acc.hi + (double)acc.lo;
+    if constexpr (HB)
+        an = sub == 0 ? an + ((double)acc_other.hi + (double)acc_other.lo) : 0.0;
 #pragma unroll
     for (int off = 16; off; off >>= 1) an += __shfl_xor_sync(0xffffffffu, an, off);
     __syncthreads();
@@ -493,7 +519,8 @@ cudaError_t launch_spectrum(const float *q, int nb, int n, int M, const FftPlan 
     SpecOut o{spec32, fstride, lp_q, lpq_fstride, lp_t, lpt_fstride, Nq, tc_ldk(M),
               lp_kind != 0, lp_kind == 3};
     // form: a cluster per image while all images' CTAs are resident at once;
-    // else 512 threads where an SM holds one CTA
+    // else half batches where an SM holds fewer than three CTAs and the images
+    // take more than one wave
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -516,13 +543,13 @@ cudaError_t launch_spectrum(const float *q, int nb, int n, int M, const FftPlan 
             break;
         }
     }
-    auto run = [&](auto kern, int threads, int width, size_t bytes) {
+    auto run = [&](auto kern, int width, size_t bytes) {
         cudaError_t er = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)bytes);
         if (er != cudaSuccess) return er;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(nb * width));
-        cfg.blockDim = dim3((unsigned)threads);
+        cfg.blockDim = dim3(kSpecThreads);
         cfg.dynamicSmemBytes = bytes;
         cfg.stream = st;
         cudaLaunchAttribute at[1];
@@ -534,11 +561,13 @@ cudaError_t launch_spectrum(const float *q, int nb, int n, int M, const FftPlan 
         return cudaLaunchKernelEx(&cfg, kern, q, n, M, plan, tw, o, prof, center, norm32, norm16,
                                   parts);
     };
-    const bool wide = smem > kSmemOptIn / 2;
+    const bool half = nsig >= 8 && smem > kSmemOptIn / 3 &&
+                      nb > sms * (smem > kSmemOptIn / 2 ? 1 : 2);
+    const size_t smem_hb = smem_of(nsig / 2);
 #define SW_SPEC_FORMS(T, NS)                                                               \
-    return S > 1    ? run(k_spectrum<T, NS, 1, true>, kSpecThreads, S, smem_cl)            \
-           : wide   ? run(k_spectrum<T, NS, 2, false>, 2 * kSpecThreads, 1, smem)          \
-                    : run(k_spectrum<T, NS, 1, false>, kSpecThreads, 1, smem)
+    return S > 1  ? run(k_spectrum<T, NS, false, true>, S, smem_cl)                        \
+           : half ? run(k_spectrum<T, NS, (NS > 4), false>, 1, smem_hb)                    \
+                  : run(k_spectrum<T, NS, false, false>, 1, smem)
     if (lp_kind == 2 || lp_kind == 3) {
         if (nsig == 16) SW_SPEC_FORMS(__half, 16);
         if (nsig == 8) SW_SPEC_FORMS(__half, 8);
