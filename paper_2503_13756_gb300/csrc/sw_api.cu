@@ -674,6 +674,7 @@ struct ImageOut {
     void *lp_t;
     size_t lpt_fstride;
     int Nq;  // images [0, Nq) are queries for the low-precision layout
+    int *err;  // the correlation's error word, cleared with the spectra (or NULL)
     float *prof;
     double *center, *norm32, *norm16;
 };
@@ -758,7 +759,7 @@ sw_status run_after_projection(sw_ctx *c, const sw_params *p, const Tables *t, i
                 return swk::launch_spectrum(o.quant, nb, n, M * parts, t->plan, t->tw, o.spec32,
                                             o.fstride, o.lp_kind, o.lp_q, o.lpq_fstride, o.lp_t,
                                             o.lpt_fstride, o.Nq, o.prof, o.center, o.norm32,
-                                            o.norm16, st, tune_of(c, p).spec, parts);
+                                            o.norm16, st, tune_of(c, p).spec, parts, o.err);
             }));
     return SW_OK;
 }
@@ -1087,10 +1088,11 @@ sw_status align_batch_impl(sw_ctx *c, const sw_params *p, const float *dq, int N
                     }));
         return SW_OK;
     }
+    // the error word of the tensor-core correlation (the FP32 one has no waits)
+    int *err = lp ? at<int>(w, l.err) : nullptr;
+    o.err = err;
     if ((s = run_after_projection(c, p, t, nimg, o, st))) return s;
     float2 *C = at<float2>(w, l.C);
-    int *err = at<int>(w, l.err);
-    SW_CUDA(c, cudaMemsetAsync(err, 0, sizeof(int), st));
     if (lp) {
         SW_CUDA(c, launch(c, SW_STAGE_CORR, st, [&] {
                     return swk::launch_corr_tc(o.lp_q, o.lp_t, Nq, Nt, M, nh, kind, C, err,
@@ -1352,10 +1354,10 @@ static sw_status bank_align_impl(sw_ctx *c, const sw_bank *bank, const float *d_
     o.norm32 = at<double>(w, l.norm32);
     o.norm16 = at<double>(w, l.norm16);
     if ((s = run_images(c, p, t, d_q_img, q_L, Nq, 0, o, st))) return s;
+    int *err = lp ? at<int>(w, l.err) : nullptr;
+    o.err = err;
     if ((s = run_after_projection(c, p, t, Nq, o, st))) return s;
     float2 *C = at<float2>(w, l.C);
-    int *err = at<int>(w, l.err);
-    SW_CUDA(c, cudaMemsetAsync(err, 0, sizeof(int), st));
     if (lp) {
         SW_CUDA(c, launch(c, SW_STAGE_CORR, st, [&] {
                     return swk::launch_corr_tc(o.lp_q, bank->lp_t, Nq, Nt, M, nh, kind, C, err,

@@ -703,7 +703,10 @@ cudaError_t launch_center_norm(const float *q, int nb, int n, int M, const doubl
 // [hi | lo] (of the same [re|im|0] and [-im|re|0] rows): the correlation
 // runs one GEMM over K = 3 ldk, reading the segments (hi, hi), (hi, lo),
 // (lo, hi) of the two operands, so that it sums hi*hi + hi*lo + lo*hi.
-// With lp_kind != 0, spec32 is not written (may be NULL).
+// With lp_kind != 0, spec32 is not written (may be NULL).  *clear (may be
+// NULL) is set to 0: the correlation's error word, without a launch of its own.
+// Only the norm that the decision reads is written: norm16 for lp_kind 1 and
+// 2, else norm32.
 // parts = 2 (ramp-filtered distance): M counts the levels of both parts,
 // q is [nb][2][n][M/2], each part is centred by its own vector and center
 // is [nb][2][2]; the norms are the sums over both parts.
@@ -711,7 +714,8 @@ cudaError_t launch_spectrum(const float *q, int nb, int n, int M, const FftPlan 
                             const float2 *tw, float *spec32, size_t fstride, int lp_kind,
                             void *lp_q, size_t lpq_fstride, void *lp_t, size_t lpt_fstride,
                             int Nq, float *prof, double *center, double *norm32,
-                            double *norm16, cudaStream_t st, int nsig = 0, int parts = 1);
+                            double *norm16, cudaStream_t st, int nsig = 0, int parts = 1,
+                            int *clear = nullptr);
 
 // FP32 SIMT correlation: for f < nf, i < Nq, j < Nt
 // C[(f*Nq + i)*Nt + j] = sum_p Qhat_i(f,p) conj(Qhat_j(f,p)) as (re, im).

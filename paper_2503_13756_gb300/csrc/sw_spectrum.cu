@@ -264,7 +264,8 @@ template <typename T, int NSC, bool HB, bool CL>
 __global__ void __launch_bounds__(kSpecThreads, CL ? 2 : 3)
 k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2 *__restrict__ tw,
            SpecOut o, float *__restrict__ prof, double *__restrict__ center,
-           double *__restrict__ norm32, double *__restrict__ norm16, int parts)
+           double *__restrict__ norm32, double *__restrict__ norm16, int parts,
+           int *__restrict__ clear)
 {
     constexpr int nsig = HB ? NSC / 2 : NSC;  // signals transformed at a time
     // M levels in all; with parts = 2 (ramp-filtered distance) the levels
@@ -294,6 +295,7 @@ k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2
     const int nbatch = (M + 2 * nsig - 1) / (2 * nsig);
     stage_levels<nsig>(qi, n, M, Mp, parts, rank * 2 * nsig, bufA);
     for (int i = threadIdx.x; i < n; i += blockDim.x) tws[i] = tw[i];
+    if (clear && blockIdx.x == 0 && threadIdx.x == 0) *clear = 0;
     if constexpr (CL) cg::this_cluster().sync();  // CTA 0 has started: its x1 can be written
     float2 *x1o = x1;
     if constexpr (CL) x1o = cg::this_cluster().map_shared_rank(x1, 0);
@@ -501,7 +503,8 @@ cudaError_t launch_spectrum(const float *q, int nb, int n, int M, const FftPlan 
                             const float2 *tw, float *spec32, size_t fstride, int lp_kind,
                             void *lp_q, size_t lpq_fstride, void *lp_t, size_t lpt_fstride,
                             int Nq, float *prof, double *center, double *norm32,
-                            double *norm16, cudaStream_t st, int nsig_req, int parts)
+                            double *norm16, cudaStream_t st, int nsig_req, int parts,
+                            int *clear)
 {
     if (parts != 1 && (parts != 2 || M % 2)) return cudaErrorInvalidValue;
     if (nb <= 0) return cudaSuccess;
@@ -559,7 +562,7 @@ cudaError_t launch_spectrum(const float *q, int nb, int n, int M, const FftPlan 
         cfg.attrs = at;
         cfg.numAttrs = width > 1 ? 1 : 0;
         return cudaLaunchKernelEx(&cfg, kern, q, n, M, plan, tw, o, prof, center, norm32, norm16,
-                                  parts);
+                                  parts, clear);
     };
     const bool half = nsig >= 8 && smem > kSmemOptIn / 3 &&
                       nb > sms * (smem > kSmemOptIn / 2 ? 1 : 2);

@@ -145,17 +145,25 @@ def load(path: str | None = None):
 
 
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
 
 
 def _stream(stream=None):
+    """The handle of the stream, or of the caller's current stream (read
+    without building a Stream object: 0.1 us instead of 3)."""
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _f32(x, device):
     import torch
+    # a small call's time is its host time: a tensor that needs no conversion
+    # skips as_tensor (3 us)
+    if (type(x) is torch.Tensor and x.dtype is torch.float32 and x.device == device
+            and x.is_contiguous()):
+        return x
     t = torch.as_tensor(x, dtype=torch.float32, device=device)
     return t.contiguous()
 
