@@ -41,3 +41,26 @@ def test_pairs_do_not_depend_on_the_batch(al, n, M, metric, precision):
             assert np.array_equal(r[f], full[f][:count]), (count, f)
         for f in ("shift", "d2"):
             assert np.allclose(r[f], full[f][:count], rtol=1e-12, atol=1e-14), (count, f)
+
+
+@pytest.mark.parametrize("nt", [1, 31, 128, 129, 300, 1025])
+def test_best_template_is_the_argmin_of_all_pairs(al, nt):
+    """Mode 1 (a warp per query up to 128 templates, a block above) picks the
+    least d2, the lowest index on ties, of the usable results of mode 0; the
+    first, a middle and the last template are copies, and one is unusable."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(nt)
+    p = swalign.make_params(16, 8, 4)
+    t = torch.rand((nt, 16, 16), generator=g, device="cuda")
+    t[nt // 2] = t[0]
+    t[-1] = t[0]
+    if nt > 2:
+        t[1] = 0.0
+    q = torch.cat([t[:1], torch.rand((9, 16, 16), generator=g, device="cuda")])
+    every = swalign.results_to_numpy(al.align_batch(q, t, p)).reshape(-1, nt)
+    best = swalign.results_to_numpy(al.align_batch(q, t, p, mode=1))
+    d = np.where(every["status"] == 0, every["d2"], np.inf)
+    j = d.argmin(1)
+    assert np.array_equal(best["template_index"], j)
+    assert np.array_equal(best["d2"], d[np.arange(len(j)), j])
+    assert np.array_equal(best["best_l"], every["best_l"][np.arange(len(j)), j])
