@@ -25,6 +25,7 @@ k_corr_simt(const float *__restrict__ X, size_t xf, const float *__restrict__ Y,
             int Nq, int Nt, int M, float2 *__restrict__ C)
 {
     __shared__ __align__(16) float qa[KP][TM], qb[KP][TM], ta[KP][TN], tb[KP][TN];
+    chain_wait();
     const int f = blockIdx.z;
     const int i0 = blockIdx.y * TM, j0 = blockIdx.x * TN;
     const float *Xf = X + (size_t)f * xf;
@@ -109,6 +110,7 @@ k_corr_few(const float *__restrict__ X, size_t xf, const float *__restrict__ Y, 
            int Nt, int M, int nf, int fb, float2 *__restrict__ C)
 {
     extern __shared__ float sm[];
+    chain_wait();
     const int M2 = 2 * M, rows = Nq + Nt, FS = rows * M2 + 1;
     const int f0 = blockIdx.x * fb, nb = min(fb, nf - f0);
     for (int fl = 0; fl < nb; ++fl) {
@@ -145,12 +147,11 @@ cudaError_t launch_corr_simt(const float *X, size_t xf, const float *Y, size_t y
     if (Nq <= 16 && Nt <= 16 && Nq * Nt <= 64 && per_f <= 48 * 1024) {
         const int fb = (int)std::max<size_t>(
             1, std::min<size_t>({48 * 1024 / per_f, (size_t)(nf + 151) / 152, (size_t)8}));
-        k_corr_few<<<(nf + fb - 1) / fb, 256, per_f * fb, st>>>(X, xf, Y, yf, Nq, Nt, M, nf, fb, C);
-        return cudaGetLastError();
+        return launch_chained(k_corr_few, dim3((nf + fb - 1) / fb), dim3(256), per_f * fb, st, 1, X,
+                              xf, Y, yf, Nq, Nt, M, nf, fb, C);
     }
     dim3 grid((Nt + TN - 1) / TN, (Nq + TM - 1) / TM, nf);
-    k_corr_simt<<<grid, 256, 0, st>>>(X, xf, Y, yf, Nq, Nt, M, C);
-    return cudaGetLastError();
+    return launch_chained(k_corr_simt, grid, dim3(256), 0, st, 1, X, xf, Y, yf, Nq, Nt, M, C);
 }
 
 }  // namespace swk

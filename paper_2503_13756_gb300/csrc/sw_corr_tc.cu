@@ -236,6 +236,7 @@ k_corr_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
     tc_fence_after();
     const uint32_t tmem = tmem_base_s;
     volatile int *abort_flag = &abort_s;
+    chain_wait();  // the setup above overlaps the previous kernel's end
 
     auto give_up = [&]() {
         *abort_flag = 1;
@@ -506,8 +507,8 @@ cudaError_t launch_tile(const void *Xq, const void *Yt, int Nq, int Nt, int M, i
                          (int)smem);
     const int tiles = nf * a.mtiles * a.ntiles;
     const int grid = tiles < num_sms ? tiles : num_sms;
-    k_corr_tc<BN, EPW, S4><<<grid, tc_threads<EPW>(), smem, st>>>(ma, mb, mc, a);
-    return cudaGetLastError();
+    return launch_chained(k_corr_tc<BN, EPW, S4>, dim3(grid), dim3(tc_threads<EPW>()), smem, st, 1,
+                          ma, mb, mc, a);
 }
 
 }  // namespace

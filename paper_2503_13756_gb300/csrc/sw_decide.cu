@@ -218,6 +218,7 @@ k_decide(DecideArgs A, FftPlan plan, const float2 *__restrict__ tw)
     const int j0 = blockIdx.y * NP;
     const int Nq = A.Nq, Nt = A.Nt;
 
+    chain_wait();
     for (int t = threadIdx.x; t < n; t += blockDim.x) tws[t] = tw[t];
     for (int p = threadIdx.x; p < M; p += blockDim.x) prof_i[p] = A.prof_q[(size_t)i * M + p];
     if (threadIdx.x < NP) {
@@ -600,6 +601,7 @@ k_decide_reg(DecideArgs A, const float2 *__restrict__ tw)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int s = warp;  // this warp's templates: j0 + 2s (real part), j0 + 2s + 1 (imaginary)
 
+    chain_wait();
     // ---- stage C(k', i, j0 .. j0 + 15), k' = 1..n/2 (row k' - 1)
     stage_block<nh>(A, i, j0, sC, tid);
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -773,6 +775,7 @@ k_best_template(const sw_result *__restrict__ all, int Nq, int Nt, sw_result *__
     __shared__ int s_j[NW], s_bad[NW];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int i = WQ == 1 ? blockIdx.x * NW + w : blockIdx.x;
+    chain_wait();
     if (i >= Nq) return;
     const sw_result *row = all + (size_t)i * Nt;
     double best = __longlong_as_double(0x7ff0000000000000ULL);
@@ -863,7 +866,8 @@ cudaError_t launch_decide(const DecideArgs &args, const FftPlan &plan, const flo
     do {                                                                                    \
         cudaFuncSetAttribute(k_decide_reg<MW, P, X, LN>,                                    \
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);       \
-        k_decide_reg<MW, P, X, LN><<<grid, kRegThreads, smem, st>>>(a, tw);                 \
+        return launch_chained(k_decide_reg<MW, P, X, LN>, grid, dim3(kRegThreads), smem, st,  \
+                              1, a, tw);                                                    \
     } while (0)
 #define SW_REG_FORMS(MW, LN)                                                                \
     do {                                                                                    \
@@ -899,7 +903,8 @@ cudaError_t launch_decide(const DecideArgs &args, const FftPlan &plan, const flo
     do {                                                                                    \
         cudaFuncSetAttribute(k_decide<NS, P, X>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                              200 * 1024);                                                   \
-        k_decide<NS, P, X><<<grid, kDecThreads, smem, st>>>(a, plan, tw);                   \
+        return launch_chained(k_decide<NS, P, X>, grid, dim3(kDecThreads), smem, st, 1, a,   \
+                              plan, tw);                                                    \
     } while (0)
     const bool plain = a.parts == 1 && a.translation && a.grid_k == 0;
     if (plain) {
@@ -925,11 +930,10 @@ cudaError_t launch_best_template(const void *all, int Nq, int Nt, void *out, cud
     const auto *res = reinterpret_cast<const sw_result *>(all);
     auto *best = reinterpret_cast<sw_result *>(out);
     if (Nt > 128)  // more than four results a lane
-        k_best_template<kBestThreads / 32><<<Nq, kBestThreads, 0, st>>>(res, Nq, Nt, best);
-    else
-        k_best_template<1><<<(Nq * 32 + kBestThreads - 1) / kBestThreads, kBestThreads, 0, st>>>(
-            res, Nq, Nt, best);
-    return cudaGetLastError();
+        return launch_chained(k_best_template<kBestThreads / 32>, dim3(Nq), dim3(kBestThreads), 0, st,
+                              1, res, Nq, Nt, best);
+    return launch_chained(k_best_template<1>, dim3((Nq * 32 + kBestThreads - 1) / kBestThreads),
+                          dim3(kBestThreads), 0, st, 1, res, Nq, Nt, best);
 }
 
 }  // namespace swk

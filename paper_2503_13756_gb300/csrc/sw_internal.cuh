@@ -432,6 +432,51 @@ __device__ __forceinline__ float2 *fft_smem(float2 *a, float2 *b, const FftPlan 
 }
 
 // ------------------------------------------------------------------------
+// Chained launches.  The kernels of a call follow one another on its stream,
+// each reading what the one before wrote; launched with programmatic stream
+// serialisation, a kernel's CTAs are scheduled while the previous kernel's
+// last ones still run, and wait here for its completion (which also makes its
+// writes visible), so the launch latency is off the critical path.  Every
+// kernel launched by launch_chained calls chain_wait before it touches
+// anything a previous kernel or call may read or write, and so the order of
+// all of them is kept: a kernel completes only after its predecessor has.
+//
+// A grid of at most kChainEarly CTAs lets the next kernel be scheduled as soon
+// as all its own CTAs run; a larger one only as they end.  Scheduled while
+// some SMs are still busy, a kernel of a few CTAs per SM fills the free SMs to
+// their limit and leaves the others short (the spectra of 338 images: 20 us of
+// 520 lost on the call).
+constexpr unsigned kChainEarly = 304;
+__device__ __forceinline__ void chain_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if ((unsigned long long)gridDim.x * gridDim.y * gridDim.z <= kChainEarly)
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Launches kern<<<grid, block, smem, st>>>(args...) in the stream's chain, as
+// clusters of `cluster` CTAs along x when cluster > 1.
+template <typename... K, typename... A>
+cudaError_t launch_chained(void (*kern)(K...), dim3 grid, dim3 block, size_t smem,
+                           cudaStream_t st, int cluster, A &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)cluster;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<K>(args)...);
+}
+
+// ------------------------------------------------------------------------
 // Launchers.  All return the launch status (cudaGetLastError).
 
 // Projection of nb images (sw_project / first stage of the alignment).

@@ -66,6 +66,7 @@ k_project(const float *__restrict__ img, int L, int srcL, int nh, int B, int G,
         s_mass = 0;
     }
     for (int i = threadIdx.x; i < G * Bp; i += blockDim.x) acc[i] = 0.f;
+    chain_wait();
 
     const float half_L1 = 0.5f * (float)(L - 1);
     const float half_B1 = 0.5f * (float)(B - 1);
@@ -219,6 +220,7 @@ k_project4(const float *__restrict__ img, int L, int srcL, int n, int B, int per
         s_bad = 0;
         s_mass = 0;
     }
+    chain_wait();
     __syncthreads();
     int bad = 0, mass = 0;
     for (int idx = threadIdx.x; idx < rowsT * S; idx += blockDim.x) {
@@ -447,9 +449,8 @@ cudaError_t launch_project(const float *img, int nb, int L, int srcL, int nh, in
             const size_t smem = sizeof(float) * (size_t)(L + 2 * kPad) * S4;
             cudaFuncSetAttribute(k_project4<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  200 * 1024);
-            k_project4<false><<<grid, kProjThreads, smem, st>>>(img, L, srcL, n, B, per, kc, cs,
-                                                                out, full_n, status, L, img2,
-                                                                nb1);
+            return launch_chained(k_project4<false>, grid, dim3(kProjThreads), smem, st, 1, img, L,
+                                  srcL, n, B, per, kc, cs, out, full_n, status, L, img2, nb1);
         } else {
             const size_t rows = (size_t)nb * (full_n ? n : nh) * B;
             cudaError_t e = cudaMemsetAsync(out, 0, sizeof(float) * rows, st);
@@ -470,9 +471,8 @@ cudaError_t launch_project(const float *img, int nb, int L, int srcL, int nh, in
     const size_t smem = sizeof(float) * ((size_t)(tg.T + 2 * kPad) * tg.S + (size_t)G * Bp);
     cudaFuncSetAttribute(k_project, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     dim3 grid((nh + G - 1) / G, nb);
-    k_project<<<grid, kProjThreads, smem, st>>>(img, L, srcL, nh, B, G, cs, out, full_n, status,
-                                                img2, nb1);
-    return cudaGetLastError();
+    return launch_chained(k_project, grid, dim3(kProjThreads), smem, st, 1, img, L, srcL, nh, B, G,
+                          cs, out, full_n, status, img2, nb1);
 }
 
 }  // namespace swk

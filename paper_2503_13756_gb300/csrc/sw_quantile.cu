@@ -172,6 +172,7 @@ k_quantiles(const float *__restrict__ proj, int n, int B, int M, float h, int le
     extern __shared__ float4 smq[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nw = blockDim.x >> 5;
+    chain_wait();
     const int nh = n / 2;
     const int nrows = mirror_out ? nh : n;  // rows computed per image
     // this warp's rows (images' rows in a row), as even a share as possible
@@ -472,6 +473,7 @@ k_center_norm(const float *__restrict__ q, int n, int M, const double2 *__restri
 {
     __shared__ double red[3][32];
     __shared__ double part[3];  // this CTA's sums: a (x, y), norm
+    chain_wait();
     cg::cluster_group cl = cg::this_cluster();
     const int S = (int)cl.num_blocks(), rank = (int)cl.block_rank();
     const int imgi = blockIdx.x / S;
@@ -587,9 +589,8 @@ cudaError_t launch_quantiles(const float *proj, int nb, int n, int B, int M, flo
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              200 * 1024);
         if (e != cudaSuccess) return e;
-        kern<<<grid, 32 * nw, smem, st>>>(proj, n, B, M, h, level_rule, half, mirror, nrow, q,
-                                          status, status_shift);
-        return cudaGetLastError();
+        return launch_chained(kern, dim3(grid), dim3(32 * nw), smem, st, 1, proj, n, B, M, h,
+                              level_rule, half, mirror, nrow, q, status, status_shift);
     };
     if (C > 12) C = 0;
     switch (C) {
@@ -619,17 +620,8 @@ cudaError_t launch_center_norm(const float *q, int nb, int n, int M, const doubl
     // cluster size) at most
     int S = 1;
     while (S < 8 && (long long)nb * S < 4 * 152) S *= 2;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(nb * S));
-    cfg.blockDim = dim3(256);
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)S;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_center_norm, q, n, M, cs64, center, norm);
+    return launch_chained(k_center_norm, dim3((unsigned)(nb * S)), dim3(256), 0, st, S, q, n, M, cs64,
+                          center, norm);
 }
 
 }  // namespace swk

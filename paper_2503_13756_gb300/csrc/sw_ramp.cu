@@ -33,6 +33,7 @@ k_ramp(const float *__restrict__ proj, int nh, int B, FftPlan plan,
     float2 *b1 = b0 + B * nsig;
     float2 *tws = b1 + B * nsig;                            // [B]
     float *tile = reinterpret_cast<float *>(tws + B);       // [2 nsig][B + 1] rows of the chunk
+    chain_wait();
     const int TS = B + 1;  // odd row stride (B is even): column reads hit distinct banks
     for (int i = threadIdx.x; i < B; i += blockDim.x) tws[i] = tw[i];
     const int img = blockIdx.x;
@@ -100,7 +101,8 @@ cudaError_t launch_ramp(const float *proj, int nb, int nh, int B, const FftPlan 
     do {                                                                                      \
         cudaFuncSetAttribute(k_ramp<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize,         \
                              200 * 1024);                                                     \
-        k_ramp<NS><<<nb, kRampThreads, smem, st>>>(proj, nh, B, plan, tw, parts);             \
+        return launch_chained(k_ramp<NS>, dim3(nb), dim3(kRampThreads), smem, st, 1, proj, nh, \
+                              B, plan, tw, parts);                                            \
     } while (0)
     if (nsig == 16) SW_RAMP_LAUNCH(16);
     else if (nsig == 8) SW_RAMP_LAUNCH(8);

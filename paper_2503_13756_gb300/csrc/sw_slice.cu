@@ -779,6 +779,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_project_slice(SliceArgs A)
             prefetch_l2(image_of(A, gi + A.pf_ahead), sizeof(float) * A.srcL * A.srcL);
     }
     for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = A.tw[i];
+    chain_wait();
     image_sync<CL>();
     int bad = 0, mass = 0;
     slice_grid<M, CL>(A, image_of(A, gi), G, tw, warp, kSliceThreads / 32, lane, bad, mass,
@@ -815,6 +816,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_project_slice_up(SliceArgs
     }
     for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = A.tw[i];
     for (int i = threadIdx.x; i < 2 * N; i += blockDim.x) tw2[i] = A.tw2[i];
+    chain_wait();
     image_sync<CL>();
     int bad = 0, mass = 0;
     slice_grid<MG, CL>(A, image_of(A, gi), G, tw, warp, kSliceThreads / 32, lane, bad, mass,
@@ -841,6 +843,7 @@ __global__ void __launch_bounds__(kBigThreads, 2) k_slice_grid(SliceArgs A)
         s_flags = 0;
     }
     for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = A.tw[i];
+    chain_wait();
     image_sync<CL>();
     extern __shared__ float stg[];  // [2][L][33] image bands (not upsampled)
     float2 *G = A.grid + (size_t)(gi - A.img_off) * slice_rows(N) * slice_stride(N);
@@ -860,6 +863,7 @@ __global__ void __launch_bounds__(kBigThreads) k_slice_tile(SliceArgs A)
     constexpr int N = 32 * M;
     constexpr int TS = kSliceTileSpan, RS = kSliceTileRS;
     __shared__ float2 T[TS * RS];
+    chain_wait();
     const int rows = slice_rows(N), S = slice_stride(N), nj = N / 2 + 1;
     const int tile = blockIdx.x;
     const int r0 = (tile / slice_tiles_x(N)) * kSliceTile, c0 = (tile % slice_tiles_x(N)) * kSliceTile;
@@ -905,6 +909,7 @@ __global__ void __launch_bounds__(kBigThreads, 2) k_slice_rows(SliceArgs A)
     float2 *tw = Xs + kBigBatch * nj;   // [N]
     for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = A.tw[i];
     const int k0 = blockIdx.x * kBigBatch;
+    chain_wait();
     const float2 *X = A.xs + ((size_t)blockIdx.y * A.nh + k0) * nj;
     const int valid = min(kBigBatch, A.nh - k0) * nj;
     for (int it = threadIdx.x; it < kBigBatch * nj; it += blockDim.x)
@@ -941,18 +946,7 @@ cudaError_t launch_cluster(K kern, int nb, int P, int threads, size_t smem, cons
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(nb * P));
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)P;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = P > 1 ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, a);
+    return launch_chained(kern, dim3((unsigned)(nb * P)), dim3((unsigned)threads), smem, st, P, a);
 }
 
 // One CTA per image, or, for fewer images than would fill the chip, a
@@ -1011,9 +1005,10 @@ cudaError_t launch_big(SliceArgs a, int nb, int chunk, cudaStream_t st)
         e = P > 1 ? launch_cluster(k_slice_grid<M, true>, cnt, P, kBigThreads, smem_grid, a, st)
                   : launch_cluster(k_slice_grid<M, false>, cnt, 1, kBigThreads, smem_grid, a, st);
         if (e != cudaSuccess) return e;
-        k_slice_tile<M><<<dim3(ntiles, cnt), kBigThreads, 0, st>>>(a);
-        k_slice_rows<M><<<dim3(nbatch, cnt), kBigThreads, smem, st>>>(a);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        e = launch_chained(k_slice_tile<M>, dim3(ntiles, cnt), dim3(kBigThreads), 0, st, 1, a);
+        if (e != cudaSuccess) return e;
+        e = launch_chained(k_slice_rows<M>, dim3(nbatch, cnt), dim3(kBigThreads), smem, st, 1, a);
+        if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }

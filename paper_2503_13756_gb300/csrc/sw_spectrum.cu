@@ -293,6 +293,7 @@ k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2
     const int img = blockIdx.x / S;
     const float *qi = q + (size_t)img * n * M;
     const int nbatch = (M + 2 * nsig - 1) / (2 * nsig);
+    chain_wait();
     stage_levels<nsig>(qi, n, M, Mp, parts, rank * 2 * nsig, bufA);
     for (int i = threadIdx.x; i < n; i += blockDim.x) tws[i] = tw[i];
     if (clear && blockIdx.x == 0 && threadIdx.x == 0) *clear = 0;
@@ -550,19 +551,9 @@ cudaError_t launch_spectrum(const float *q, int nb, int n, int M, const FftPlan 
         cudaError_t er = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)bytes);
         if (er != cudaSuccess) return er;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(nb * width));
-        cfg.blockDim = dim3(kSpecThreads);
-        cfg.dynamicSmemBytes = bytes;
-        cfg.stream = st;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = (unsigned)width;
-        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = width > 1 ? 1 : 0;
-        return cudaLaunchKernelEx(&cfg, kern, q, n, M, plan, tw, o, prof, center, norm32, norm16,
-                                  parts, clear);
+        return launch_chained(kern, dim3((unsigned)(nb * width)), dim3(kSpecThreads), bytes, st,
+                              width, q, n, M, plan, tw, o, prof, center, norm32, norm16, parts,
+                              clear);
     };
     const bool half = nsig >= 8 && smem > kSmemOptIn / 3 &&
                       nb > sms * (smem > kSmemOptIn / 2 ? 1 : 2);
