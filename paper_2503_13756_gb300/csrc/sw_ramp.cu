@@ -36,6 +36,7 @@ k_ramp(const float *__restrict__ proj, int nh, int B, FftPlan plan,
     chain_wait();
     const int TS = B + 1;  // odd row stride (B is even): column reads hit distinct banks
     for (int i = threadIdx.x; i < B; i += blockDim.x) tws[i] = tw[i];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int img = blockIdx.x;
     const float *U = proj + (size_t)img * nh * B;
     float *Pp = parts + (size_t)img * 2 * nh * B;  // part 0 (positive)
@@ -45,9 +46,11 @@ k_ramp(const float *__restrict__ proj, int nh, int B, FftPlan plan,
         const int rows = min(2 * nsig, nh - r0);
         // ---- load the chunk's rows (coalesced), then pack: signal s =
         // rows (2s, 2s + 1) as (re, im), element-major for the FFT
-        for (int e = threadIdx.x; e < 2 * nsig * B; e += blockDim.x) {
-            const int r = e / B, b = e - r * B;
-            tile[r * TS + b] = r < rows ? U[(size_t)(r0 + r) * B + b] : 0.f;
+        // (a warp per row: no division by B per element)
+        for (int r = warp; r < 2 * nsig; r += kRampThreads / 32) {
+            const float *row = U + (size_t)(r0 + r) * B;
+#pragma unroll 4
+            for (int b = lane; b < B; b += 32) tile[r * TS + b] = r < rows ? __ldg(row + b) : 0.f;
         }
         __syncthreads();
         for (int t = threadIdx.x; t < B * nsig; t += blockDim.x) {
@@ -72,11 +75,14 @@ k_ramp(const float *__restrict__ proj, int nh, int B, FftPlan plan,
             tile[(2 * sg + 1) * TS + b] = v.y;
         }
         __syncthreads();
-        for (int e = threadIdx.x; e < rows * B; e += blockDim.x) {
-            const int r = e / B, b = e - r * B;
-            const float v = tile[r * TS + b];
-            Pp[(size_t)(r0 + r) * B + b] = fmaxf(v, 0.f);
-            Pm[(size_t)(r0 + r) * B + b] = fmaxf(-v, 0.f);
+        for (int r = warp; r < rows; r += kRampThreads / 32) {
+            float *pp = Pp + (size_t)(r0 + r) * B, *pm = Pm + (size_t)(r0 + r) * B;
+#pragma unroll 4
+            for (int b = lane; b < B; b += 32) {
+                const float v = tile[r * TS + b];
+                pp[b] = fmaxf(v, 0.f);
+                pm[b] = fmaxf(-v, 0.f);
+            }
         }
         __syncthreads();
     }
