@@ -179,15 +179,15 @@ __device__ __forceinline__ void slice_grid(const SliceArgs &A, const float *__re
 {
     const int P = CL ? (int)cg::this_cluster().num_blocks() : 1;
     const int rank = CL ? (int)cg::this_cluster().block_rank() : 0;
-    // phase A's value of a kept row: to the CTA that transforms the row
-    auto put_row = [&](int i, int idx, float2 val) {
-        if constexpr (CL && SHARED) cg::this_cluster().map_shared_rank(G, i & (P - 1))[idx] = val;
-        else G[idx] = val;
-    };
     constexpr int N = 32 * M;
     const int L = A.L, half = L / 2;
     const int rows = slice_rows(N), S = slice_stride(N), lo = slice_lo(N);
     const int nleft = slice_left(N), nright = slice_right(N);
+    // Between the phases row i holds its columns from `turn` on (grid in shared
+    // memory): the lanes of a column pair's store hold rows M apart, which lie
+    // on four banks of the final layout (S = 1 mod 16); turned by the output's
+    // 32-point index b, each quarter-warp's 16-byte stores hit eight.
+    auto turn = [&](int i, int b) { return SHARED ? (2 * (b >> 2) - i) & 15 : 0; };
     // ---- A: one warp per column pair (c, c+1): FFT along r', kept rows.
     // fetch(r) gives the pixels (r, c) and (r, c + 1).
     auto read_pair = [&](float2 (&v)[M], int c, auto fetch) {
@@ -232,10 +232,19 @@ __device__ __forceinline__ void slice_grid(const SliceArgs &A, const float *__re
             const int i = wrap_n(k1 + kb - lo, N);  // kept row of l2 = kout (mod N)
             if (i < rows) {
                 // column c: (Z + conj Z(-l2)) / 2; column c + 1: (Z - conj Z(-l2)) / (2i)
-                put_row(i, i * S + c, make_float2(0.5f * (Z.x + Zc.x), 0.5f * (Z.y + Zc.y)));
-                if (c + 1 < L)
-                    put_row(i, i * S + c + 1,
-                            make_float2(0.5f * (Z.y - Zc.y), -0.5f * (Z.x - Zc.x)));
+                const float2 x0 = make_float2(0.5f * (Z.x + Zc.x), 0.5f * (Z.y + Zc.y));
+                const float2 x1 = make_float2(0.5f * (Z.y - Zc.y), -0.5f * (Z.x - Zc.x));
+                if constexpr (SHARED) {
+                    // to the CTA that transforms the row (column L of an odd L is
+                    // not read); i S + turn + c is even
+                    float2 *Gr = G;
+                    if constexpr (CL) Gr = cg::this_cluster().map_shared_rank(G, i & (P - 1));
+                    *reinterpret_cast<float4 *>(Gr + i * S + turn(i, brev5(lane)) + c) =
+                        make_float4(x0.x, x0.y, x1.x, x1.y);
+                } else {
+                    G[i * S + c] = x0;
+                    if (c + 1 < L) G[i * S + c + 1] = x1;
+                }
             }
         }
     };
@@ -248,11 +257,12 @@ __device__ __forceinline__ void slice_grid(const SliceArgs &A, const float *__re
     auto rows_phase = [&] {
         for (int i = rank + P * warp; i < rows; i += P * nw) {
             float2 v[M];
+            const float2 *Gi = G + i * S + turn(i, wrap_n(i + lo, N) / M);
 #pragma unroll
             for (int n1 = 0; n1 < M; ++n1) {
                 const int n = 32 * n1 + lane;
                 const int c = (n < N / 2 ? n : n - N) + half;
-                v[n1] = (c >= 0 && c < L) ? G[i * S + c] : make_float2(0.f, 0.f);
+                v[n1] = (c >= 0 && c < L) ? Gi[c] : make_float2(0.f, 0.f);
             }
             __syncwarp();
             warp_ifft<M>(v, tw, lane);
