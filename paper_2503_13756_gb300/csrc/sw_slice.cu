@@ -186,8 +186,12 @@ __device__ __forceinline__ void slice_grid(const SliceArgs &A, const float *__re
     // Between the phases row i holds its columns from `turn` on (grid in shared
     // memory): the lanes of a column pair's store hold rows M apart, which lie
     // on four banks of the final layout (S = 1 mod 16); turned by the output's
-    // 32-point index b, each quarter-warp's 16-byte stores hit eight.
-    auto turn = [&](int i, int b) { return SHARED ? (2 * (b >> 2) - i) & 15 : 0; };
+    // 32-point index b, each quarter-warp's 16-byte stores hit eight.  In global
+    // memory a row starts one column later where that aligns it to 16 bytes.
+    auto turn = [&](int i, int b) {
+        if constexpr (SHARED) return (2 * (b >> 2) - i) & 15;
+        else return (int)(reinterpret_cast<uintptr_t>(G + i * S) >> 3) & 1;
+    };
     // ---- A: one warp per column pair (c, c+1): FFT along r', kept rows.
     // fetch(r) gives the pixels (r, c) and (r, c + 1).
     auto read_pair = [&](float2 (&v)[M], int c, auto fetch) {
@@ -234,17 +238,13 @@ __device__ __forceinline__ void slice_grid(const SliceArgs &A, const float *__re
                 // column c: (Z + conj Z(-l2)) / 2; column c + 1: (Z - conj Z(-l2)) / (2i)
                 const float2 x0 = make_float2(0.5f * (Z.x + Zc.x), 0.5f * (Z.y + Zc.y));
                 const float2 x1 = make_float2(0.5f * (Z.y - Zc.y), -0.5f * (Z.x - Zc.x));
-                if constexpr (SHARED) {
-                    // to the CTA that transforms the row (column L of an odd L is
-                    // not read); i S + turn + c is even
-                    float2 *Gr = G;
-                    if constexpr (CL) Gr = cg::this_cluster().map_shared_rank(G, i & (P - 1));
-                    *reinterpret_cast<float4 *>(Gr + i * S + turn(i, brev5(lane)) + c) =
-                        make_float4(x0.x, x0.y, x1.x, x1.y);
-                } else {
-                    G[i * S + c] = x0;
-                    if (c + 1 < L) G[i * S + c + 1] = x1;
-                }
+                // to the CTA that transforms the row (column L of an odd L is not
+                // read); i S + turn + c is even
+                float2 *Gr = G;
+                if constexpr (CL && SHARED)
+                    Gr = cg::this_cluster().map_shared_rank(G, i & (P - 1));
+                *reinterpret_cast<float4 *>(Gr + i * S + turn(i, brev5(lane)) + c) =
+                    make_float4(x0.x, x0.y, x1.x, x1.y);
             }
         }
     };
