@@ -434,24 +434,22 @@ __device__ __forceinline__ float2 *fft_smem(float2 *a, float2 *b, const FftPlan 
 // ------------------------------------------------------------------------
 // Chained launches.  The kernels of a call follow one another on its stream,
 // each reading what the one before wrote; launched with programmatic stream
-// serialisation, a kernel's CTAs are scheduled while the previous kernel's
-// last ones still run, and wait here for its completion (which also makes its
-// writes visible), so the launch latency is off the critical path.  Every
-// kernel launched by launch_chained calls chain_wait before it touches
-// anything a previous kernel or call may read or write, and so the order of
-// all of them is kept: a kernel completes only after its predecessor has.
+// serialisation, a kernel is prepared while its predecessor runs, its CTAs
+// start as the last of the predecessor's end, and they wait here for its
+// completion (which also makes its writes visible): 1 to 2 us less at every
+// kernel boundary (a 64 x 64 pair 63 -> 53 us, a request of three images 170 ->
+// 156 us).  Every kernel launched by launch_chained calls chain_wait before it
+// touches anything a previous kernel or call may read or write, and so the
+// order of all of them is kept: a kernel completes only after its predecessor.
 //
-// A grid of at most kChainEarly CTAs lets the next kernel be scheduled as soon
-// as all its own CTAs run; a larger one only as they end.  Scheduled while
-// some SMs are still busy, a kernel of a few CTAs per SM fills the free SMs to
-// their limit and leaves the others short (the spectra of 338 images: 20 us of
-// 520 lost on the call).
-constexpr unsigned kChainEarly = 304;
+// No kernel lets its successor in before that (griddepcontrol.
+// launch_dependents): the waiting CTAs then hold registers and shared memory
+// that other streams' kernels could use (a batch of five sizes in concurrent
+// branches, 320 images: 476 against 426 us), and kernels of a few CTAs per SM
+// crowd the SMs that are free first (the spectra of 338 images: 20 us lost).
 __device__ __forceinline__ void chain_wait()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if ((unsigned long long)gridDim.x * gridDim.y * gridDim.z <= kChainEarly)
-        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Launches kern<<<grid, block, smem, st>>>(args...) in the stream's chain, as

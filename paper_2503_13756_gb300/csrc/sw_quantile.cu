@@ -617,9 +617,10 @@ cudaError_t launch_center_norm(const float *q, int nb, int n, int M, const doubl
 {
     if (nb <= 0) return cudaSuccess;
     // CTAs per image: enough for four on each of 152 SMs, eight (the portable
-    // cluster size) at most
+    // cluster size) at most, and at least four rows to a warp (below that the
+    // reductions cost more than the rows: 151 images at n = 96)
     int S = 1;
-    while (S < 8 && (long long)nb * S < 4 * 152) S *= 2;
+    while (S < 8 && (long long)nb * S < 4 * 152 && 64 * S <= n) S *= 2;
     return launch_chained(k_center_norm, dim3((unsigned)(nb * S)), dim3(256), 0, st, S, q, n, M, cs64,
                           center, norm);
 }
