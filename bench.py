@@ -59,9 +59,9 @@ def slice_flops_per_image(Lc, n, B):
 
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per 128 x 128 image
-# of the slice projector kernel, from one ncu capture of a 512-image launch
-# (33,824,768 + 40,143,104 bytes); None once that kernel changes.
-SLICE_DRAM_BYTES_PER_IMAGE = 73967872 / 512
+# of the slice projector kernel, from one ncu capture of a 1088-image launch
+# (71,559,680 + 52,966,656 bytes); None once that kernel changes.
+SLICE_DRAM_BYTES_PER_IMAGE = 124526336 / 1088
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per 128 x 128 image
 # of the four-angle projection kernel, from one ncu capture of its 2112-image
 # launch (2048 queries and 64 templates in one launch: 277,210,112 bytes);
@@ -906,7 +906,7 @@ def main():
             "achieved": smem_ach, "peak": smem_peak, "unit": "TB/s", "frac": smem_ach / smem_peak,
             "tap_bytes_per_image": tap_bytes,
             "note": "tap loads only; the FFT exchanges and stores add the rest of the pipe's "
-                    "load (ncu: L1/shared 89% of peak)"}
+                    "load (ncu: L1/shared 70% of peak)"}
     elif dom == "project":
         flops = args.steps * nimg * L * L * (N_THETA // 2) * PROJ_FLOPS_PER_CELL_ANGLE
         achieved = flops / (stages[dom][0] / 1e3) / 1e12

@@ -44,10 +44,10 @@
 //     inverse FFT; the real and imaginary parts are the two rows, staged in
 //     the warp's own slice-sample rows so that the row stores coalesce.
 // Two arrangements:
-//  - L <= 128 (k_project_slice): one CTA of 32 warps per image with the whole
-//    grid in shared memory (175 KB at L = 128); 64-angle batches; the
-//    targets grouped so that each tap load of a half-warp hits 16 distinct
-//    banks (one pass).
+//  - L <= 128 (k_project_slice): one CTA of 32 warps per image (a cluster of
+//    them when there are few images) with the whole grid in shared memory
+//    (175 KB at L = 128); 64-angle batches; the targets grouped so that each
+//    tap load of a half-warp hits 16 distinct banks (one pass).
 //  - 128 < L <= 256 (k_slice_grid, k_slice_tile, k_slice_rows): the grid of
 //    a chunk of images is built in a global scratch buffer (one CTA of 16
 //    warps per image, phases A and B, the image staged in 32-column bands);
