@@ -239,7 +239,9 @@ __device__ __forceinline__ void slice_grid(const SliceArgs &A, const float *__re
                 const float2 x0 = make_float2(0.5f * (Z.x + Zc.x), 0.5f * (Z.y + Zc.y));
                 const float2 x1 = make_float2(0.5f * (Z.y - Zc.y), -0.5f * (Z.x - Zc.x));
                 // to the CTA that transforms the row (column L of an odd L is not
-                // read); i S + turn + c is even
+                // read); one 16-byte store: G starts on 16 bytes in shared memory
+                // (declared so by the kernels) and i S + turn + c is even there;
+                // in global memory turn makes the address a multiple of 16
                 float2 *Gr = G;
                 if constexpr (CL && SHARED)
                     Gr = cg::this_cluster().map_shared_rank(G, i & (P - 1));
@@ -773,8 +775,9 @@ template <int M, bool CL>
 __global__ void __launch_bounds__(kSliceThreads, 1) k_project_slice(SliceArgs A)
 {
     constexpr int N = 32 * M;
-    extern __shared__ float2 sms[];
+    extern __shared__ __align__(16) float2 sms[];
     const int nj = N / 2 + 1;
+    static_assert(__alignof__(sms) >= 16, "the grid takes 16-byte stores");
     float2 *G = sms;                                        // [rows][S] grid
     float2 *Xs = G + slice_rows(N) * slice_stride(N);       // [kSliceBatch][nj]
     float2 *tw = Xs + kSliceBatch * nj;                     // [N]
@@ -811,7 +814,8 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_project_slice_up(SliceArgs
 {
     constexpr int N = 32 * MG;
     constexpr int nj = N + 1;
-    extern __shared__ float2 sms[];
+    extern __shared__ __align__(16) float2 sms[];
+    static_assert(__alignof__(sms) >= 16, "the grid takes 16-byte stores");
     float2 *G = sms;                                        // [rows][S] grid
     float2 *Xs = G + slice_rows(N) * slice_stride(N);       // [kUpBatch][nj]
     float2 *tw = Xs + kUpBatch * nj;                        // [N]
@@ -914,7 +918,7 @@ __global__ void __launch_bounds__(kBigThreads, 2) k_slice_rows(SliceArgs A)
 {
     constexpr int N = 32 * M;
     constexpr int nj = N / 2 + 1;
-    extern __shared__ float2 sms[];
+    extern __shared__ __align__(16) float2 sms[];
     float2 *Xs = sms;                   // [kBigBatch][nj]
     float2 *tw = Xs + kBigBatch * nj;   // [N]
     for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = A.tw[i];
