@@ -310,11 +310,15 @@ sw_status fail(sw_ctx *c, sw_status s, const char *fmt, ...)
     return s;
 }
 
+// Reports a failed runtime call, and clears the last error: it belongs to this
+// call and must not fail a later one.
 #define SW_CUDA(ctx, call)                                                                   \
     do {                                                                                     \
         cudaError_t e_ = (call);                                                             \
-        if (e_ != cudaSuccess)                                                               \
+        if (e_ != cudaSuccess) {                                                             \
+            cudaGetLastError();                                                              \
             return fail((ctx), SW_ERR_CUDA, "%s failed: %s", #call, cudaGetErrorString(e_)); \
+        }                                                                                    \
     } while (0)
 
 // Runs one kernel launch `fn` on `st`, counting it and, when profiling,

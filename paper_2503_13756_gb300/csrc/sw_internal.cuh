@@ -471,7 +471,10 @@ cudaError_t launch_chained(void (*kern)(K...), dim3 grid, dim3 block, size_t sme
     at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = cluster > 1 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, kern, static_cast<K>(args)...);
+    cudaLaunchKernelEx(&cfg, kern, static_cast<K>(args)...);
+    // the launch's status, taken: left in place, it would be found by the next
+    // check of the last error, in a call that has done nothing wrong
+    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------------
