@@ -797,8 +797,11 @@ sw_status sw_create(int device, sw_ctx **out)
     sw_ctx *c = new (std::nothrow) sw_ctx;
     if (!c) return SW_ERR_OOM;
     c->device = device;
+    // (the launch rules' view of the device is asked for here, outside any capture)
+    const swk::DeviceForm *form;
     if (cudaSetDevice(device) != cudaSuccess ||
-        cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
+        cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+        swk::device_form(&form) != cudaSuccess) {
         cudaGetLastError();
         delete c;
         return SW_ERR_CUDA;

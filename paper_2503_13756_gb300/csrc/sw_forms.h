@@ -1,0 +1,119 @@
+// sw_forms.h -- which form of a kernel a launch takes, from the call's sizes
+// and the device alone.  Host code without CUDA, so that the rules can be
+// checked without a device.
+#pragma once
+
+#include <algorithm>
+#include <cstddef>
+
+namespace swk {
+
+// What the rules ask of the device: its multiprocessors, and how many clusters
+// of w CTAs it holds at once where p CTAs fit an SM (clusters[p - 1][w], p = 1,
+// 2, w = 1..8; 0: none).  The runtime knows the latter: a cluster stays within
+// a GPC, and the GPCs of a part differ (a GB300 of 152 SMs holds 76, 46, 36,
+// 28, 23, 15 and 15 clusters of 2..8 CTAs of one per SM, not 8 floor(19 / w)).
+struct DeviceForm {
+    int sms;
+    int clusters[2][9];
+};
+
+// CTAs per image (a power of two, at most the portable cluster size 8) of the
+// slice projector with the grid in shared memory, one CTA per SM: the widest
+// cluster with room for all nb images at once.  A cluster too many runs after
+// the others: 16 images in clusters of 8, of which 15 are resident, took twice
+// the time of 15 (L = 64, n = 8: 25 us, 15 us in clusters of 4).
+inline int slice_cluster(int nb, const DeviceForm &d)
+{
+    for (int P = 8; P > 1; P /= 2)
+        if (nb <= d.clusters[0][P]) return P;
+    return 1;
+}
+
+// The same for its global grid build, two CTAs per SM.  Two CTAs of an SM
+// share its pipes, so clusters of 8 and 4 gain until they fill two thirds of
+// their places (of the time on one CTA per image, L = 160..256: 20 images 0.49
+// in clusters of 8 and 0.51 in clusters of 4, 36 images 0.57 and 0.55; 37
+// images 0.70 in clusters of 4 and 2, 72 images 0.78 and 0.75; 152 images 0.99
+// in clusters of 2).
+inline int slice_grid_cluster(int nb, const DeviceForm &d)
+{
+    for (int P = 8; P > 2; P /= 2)
+        if (3 * nb <= 2 * d.clusters[1][P]) return P;
+    return nb <= d.clusters[1][2] ? 2 : 1;
+}
+
+// The angle spectra (k_spectrum).
+constexpr int kSpecThreads = 256;
+constexpr size_t kSmemOptIn = 227 * 1024 - 512;  // dynamic shared memory of a CTA, beside the static
+
+struct SpectrumForm {
+    int nsig;      // signals per FFT batch
+    int cluster;   // CTAs per image
+    bool half;     // half batches
+    size_t smem;   // dynamic shared memory of a CTA
+};
+
+// Form for nb images of n angles and M levels; false if an image does not fit
+// a CTA.  nsig_req: a requested batch width (0: none).  zeros: elements of zero
+// padding written per image (the low-precision rows').
+inline bool spectrum_form(int nb, int n, int M, int nsig_req, long long zeros, const DeviceForm &d,
+                          SpectrumForm *f)
+{
+    // signals per FFT batch: 16 by default, 8 at n = 1024; a requested
+    // width is taken when its buffers fit (2 n nsig complex values)
+    int nsig = n <= 512 ? 16 : 8;
+    if ((nsig_req == 4 || nsig_req == 8 || nsig_req == 16) && (size_t)n * nsig_req <= 8192)
+        nsig = nsig_req;
+    // two batch buffers (the staged input and the FFT's other buffer),
+    // within the 227 KB a CTA can hold
+    auto smem_of = [&](int ns) { return 8 * ((size_t)2 * n * ns + M + n); };
+    while (nsig > 4 && smem_of(nsig) > kSmemOptIn) nsig /= 2;
+    const size_t smem = smem_of(nsig);
+    if (smem > kSmemOptIn) return false;
+    *f = SpectrumForm{nsig, 1, false, smem};
+    const int nbatch = (M + 2 * nsig - 1) / (2 * nsig);
+
+    // A cluster per image where it is expected to save a tenth of the time, by
+    // the times of a launch in us on a GB300 (fitted at n = 8..1024, M =
+    // 64..1024; 90% of 11658 measured launches within 10% below and 7% above): 7.5 + b
+    // nbatch + z with a CTA per image, b the time of a batch and z that of the
+    // padding; 5 + 5 + 0.86 b ceil(nbatch / w) + 0.29 b nbatch + z / w in
+    // clusters of w CTAs (two barriers, the longest CTA's batches, the ordered
+    // sum of the terms), the batches 1.16 times longer where CTAs share an SM,
+    // and all but the launch again for every further set of resident clusters:
+    // 48 images at n = 360, M = 256 take 65 us alone, 51 us in clusters of 2, and
+    // 79 us in clusters of 3, of which 46 are resident.
+    const double b = nsig / 16.0 * (nsig == 16 ? 1.0 + 0.0168 * n : 3.5 + 0.0156 * n) *
+                     (M & 1 ? 1.5 : 1.0);  // odd M: copies and stores level by level
+    const double z = 0.0012 * (double)zeros;
+    const size_t per_batch = 8 * (size_t)((n / 2) / (kSpecThreads / nsig) + 1) * kSpecThreads;
+    double best = 0.9 * (7.5 + b * nbatch + z);
+    for (int w = 2; w <= std::min(8, nbatch) && nb <= d.sms; ++w) {
+        const int per = (nbatch + w - 1) / w;
+        const size_t need = smem + per_batch * per;
+        const int fit = need > kSmemOptIn ? 0 : d.clusters[need <= kSmemOptIn / 2 ? 1 : 0][w];
+        if (fit == 0) continue;
+        const int sets = (nb + fit - 1) / fit;
+        const double shared = std::min(nb, fit) * w > d.sms ? 1.16 : 1.0;
+        const double t = 5 + sets * (5 + shared * b * (0.86 * per + 0.29 * nbatch) + z / w);
+        if (t < best) {
+            best = t;
+            f->cluster = w;
+            f->smem = need;
+        }
+    }
+    if (f->cluster > 1) return true;
+
+    // Half batches where an SM holds fewer than three CTAs and the images take
+    // more than one wave.
+    const bool half = nsig >= 8 && smem > kSmemOptIn / 3 &&
+                      nb > d.sms * (smem > kSmemOptIn / 2 ? 1 : 2);
+    if (half) {
+        f->half = true;
+        f->smem = smem_of(nsig / 2);
+    }
+    return true;
+}
+
+}  // namespace swk

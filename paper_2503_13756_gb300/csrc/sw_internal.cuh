@@ -477,6 +477,11 @@ cudaError_t launch_chained(void (*kern)(K...), dim3 grid, dim3 block, size_t sme
     return cudaGetLastError();
 }
 
+// The launch rules' view of the current device (sw_forms.h), asked of the
+// runtime once per device and kept for the process.
+struct DeviceForm;
+cudaError_t device_form(const DeviceForm **out);
+
 // ------------------------------------------------------------------------
 // Launchers.  All return the launch status (cudaGetLastError).
 

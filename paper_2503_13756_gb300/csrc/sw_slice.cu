@@ -61,6 +61,7 @@
 
 #include <cooperative_groups.h>
 
+#include "sw_forms.h"
 #include "sw_internal.cuh"
 
 namespace swk {
@@ -933,26 +934,6 @@ __global__ void __launch_bounds__(kBigThreads, 2) k_slice_rows(SliceArgs A)
                                  threadIdx.x & 31);
 }
 
-// Multiprocessors of the current device.
-cudaError_t sm_count(int *sms)
-{
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    return e != cudaSuccess ? e : cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
-}
-
-// CTAs per image (a power of two, at most the portable cluster size 8) for nb
-// images where per_sm CTAs fit an SM: the widest cluster with room for all
-// images at once.  A cluster stays within one of the (at least eight) GPCs,
-// so one of 8 is counted against sms / 8 SMs a GPC.
-int cluster_width(int nb, int sms, int per_sm)
-{
-    const int gpc = sms / 8 * per_sm;  // CTA slots of a GPC
-    for (int P = 8; P > 1; P /= 2)
-        if (nb <= 8 * (gpc / P)) return P;
-    return 1;
-}
-
 template <typename K>
 cudaError_t launch_cluster(K kern, int nb, int P, int threads, size_t smem, const SliceArgs &a,
                            cudaStream_t st)
@@ -971,11 +952,11 @@ cudaError_t launch_cluster(K kern, int nb, int P, int threads, size_t smem, cons
 template <int M>
 cudaError_t launch_small(SliceArgs a, int nb, cudaStream_t st)
 {
-    int sms = 0;
-    cudaError_t e = sm_count(&sms);
+    const DeviceForm *dev;
+    cudaError_t e = device_form(&dev);
     if (e != cudaSuccess) return e;
-    a.pf_ahead = sms;  // resident CTAs: one per SM
-    const int P = cluster_width(nb, sms, 1);
+    a.pf_ahead = dev->sms;  // resident CTAs: one per SM
+    const int P = slice_cluster(nb, *dev);
     const size_t smem = slice_smem_bytes(32 * M);
     return P > 1 ? launch_cluster(k_project_slice<M, true>, nb, P, kSliceThreads, smem, a, st)
                  : launch_cluster(k_project_slice<M, false>, nb, 1, kSliceThreads, smem, a, st);
@@ -984,11 +965,11 @@ cudaError_t launch_small(SliceArgs a, int nb, cudaStream_t st)
 template <int MG>
 cudaError_t launch_up(SliceArgs a, int nb, cudaStream_t st)
 {
-    int sms = 0;
-    cudaError_t e = sm_count(&sms);
+    const DeviceForm *dev;
+    cudaError_t e = device_form(&dev);
     if (e != cudaSuccess) return e;
-    a.pf_ahead = sms;
-    const int P = cluster_width(nb, sms, 1);
+    a.pf_ahead = dev->sms;
+    const int P = slice_cluster(nb, *dev);
     const size_t smem = slice_up_smem_bytes(64 * MG);
     return P > 1 ? launch_cluster(k_project_slice_up<MG, true>, nb, P, kSliceThreads, smem, a, st)
                  : launch_cluster(k_project_slice_up<MG, false>, nb, 1, kSliceThreads, smem, a, st);
@@ -1006,8 +987,8 @@ cudaError_t launch_big(SliceArgs a, int nb, int chunk, cudaStream_t st)
     if (e != cudaSuccess) return e;
     // two 32-column bands of the image (rows 33 floats apart) when not upsampled
     const size_t smem_grid = a.srcL == a.L ? sizeof(float) * 2 * (size_t)a.L * 33 : 0;
-    int sms = 0;
-    if ((e = sm_count(&sms)) != cudaSuccess) return e;
+    const DeviceForm *dev;
+    if ((e = device_form(&dev)) != cudaSuccess) return e;
     // chunks of equal size (at most `chunk`): no small last chunk whose
     // launches would leave most SMs idle
     const int nchunks = (nb + chunk - 1) / chunk;
@@ -1015,7 +996,7 @@ cudaError_t launch_big(SliceArgs a, int nb, int chunk, cudaStream_t st)
     for (int i0 = 0; i0 < nb; i0 += chunk) {
         const int cnt = std::min(chunk, nb - i0);
         a.img_off = i0;
-        const int P = cluster_width(cnt, sms, 2);
+        const int P = slice_grid_cluster(cnt, *dev);
         e = P > 1 ? launch_cluster(k_slice_grid<M, true>, cnt, P, kBigThreads, smem_grid, a, st)
                   : launch_cluster(k_slice_grid<M, false>, cnt, 1, kBigThreads, smem_grid, a, st);
         if (e != cudaSuccess) return e;

@@ -23,17 +23,13 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
-#include <algorithm>
-
+#include "sw_forms.h"
 #include "sw_internal.cuh"
 
 namespace swk {
 namespace {
 
 namespace cg = cooperative_groups;
-
-constexpr int kSpecThreads = 256;
-constexpr size_t kSmemOptIn = 227 * 1024 - 512;  // dynamic shared memory of a CTA, beside the static
 
 template <typename T>
 __device__ __forceinline__ T to_lp(float x);
@@ -509,66 +505,36 @@ cudaError_t launch_spectrum(const float *q, int nb, int n, int M, const FftPlan 
 {
     if (parts != 1 && (parts != 2 || M % 2)) return cudaErrorInvalidValue;
     if (nb <= 0) return cudaSuccess;
-    // signals per FFT batch: 16 by default, 8 at n = 1024; a requested
-    // width is taken when its buffers fit (2 n nsig complex values)
-    int nsig = n <= 512 ? 16 : 8;
-    if ((nsig_req == 4 || nsig_req == 8 || nsig_req == 16) && (size_t)n * nsig_req <= 8192)
-        nsig = nsig_req;
-    // two batch buffers (the staged input and the FFT's other buffer),
-    // within the 227 KB a CTA can hold
-    auto smem_of = [&](int ns) { return sizeof(float2) * ((size_t)2 * n * ns + M + n); };
-    while (nsig > 4 && smem_of(nsig) > kSmemOptIn) nsig /= 2;
-    const size_t smem = smem_of(nsig);
-    if (smem > kSmemOptIn) return cudaErrorInvalidValue;
+    const DeviceForm *dev;
+    cudaError_t e = device_form(&dev);
+    if (e != cudaSuccess) return e;
     SpecOut o{spec32, fstride, lp_q, lpq_fstride, lp_t, lpt_fstride, Nq, tc_ldk(M),
               lp_kind != 0, lp_kind == 3};
-    // form: a cluster per image while all images' CTAs are resident at once;
-    // else half batches where an SM holds fewer than three CTAs and the images
-    // take more than one wave
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    const int nbatch = (M + 2 * nsig - 1) / (2 * nsig);
-    const size_t per_batch = sizeof(float2) * (size_t)((n / 2) / (kSpecThreads / nsig) + 1) *
-                             kSpecThreads;
-    int S = 1;
-    size_t smem_cl = smem;
-    for (int w = std::min(8, nbatch); w > 1; --w) {
-        const size_t need = smem + per_batch * ((nbatch + w - 1) / w);
-        const int per_sm = need <= kSmemOptIn / 2 ? 2 : 1;
-        // (a cluster stays within one of the at least eight GPCs)
-        // (a narrow cluster loses its gain to the two barriers and the ordered
-        // sum: 80 images of four batches take 28 us on clusters of 3 or alone)
-        if (nbatch - (nbatch + w - 1) / w < 3) break;
-        if (need <= kSmemOptIn && nb <= 8 * (sms / 8 * per_sm / w)) {
-            S = w;
-            smem_cl = need;
-            break;
-        }
-    }
-    auto run = [&](auto kern, int width, size_t bytes) {
+    // zeros of a template's two rows where there are templates, of a query's one elsewhere
+    const long long zeros = o.lp ? (long long)(n / 2) * (o.ldk - 2 * M) * (o.split ? 2 : 1) *
+                                       (Nq < nb ? 2 : 1)
+                                 : 0;
+    SpectrumForm f;
+    if (!spectrum_form(nb, n, M, nsig_req, zeros, *dev, &f)) return cudaErrorInvalidValue;
+    auto run = [&](auto kern) {
         cudaError_t er = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)bytes);
+                                              (int)f.smem);
         if (er != cudaSuccess) return er;
-        return launch_chained(kern, dim3((unsigned)(nb * width)), dim3(kSpecThreads), bytes, st,
-                              width, q, n, M, plan, tw, o, prof, center, norm32, norm16, parts,
-                              clear);
+        return launch_chained(kern, dim3((unsigned)(nb * f.cluster)), dim3(kSpecThreads), f.smem,
+                              st, f.cluster, q, n, M, plan, tw, o, prof, center, norm32, norm16,
+                              parts, clear);
     };
-    const bool half = nsig >= 8 && smem > kSmemOptIn / 3 &&
-                      nb > sms * (smem > kSmemOptIn / 2 ? 1 : 2);
-    const size_t smem_hb = smem_of(nsig / 2);
-#define SW_SPEC_FORMS(T, NS)                                                               \
-    return S > 1  ? run(k_spectrum<T, NS, false, true>, S, smem_cl)                        \
-           : half ? run(k_spectrum<T, NS, (NS > 4), false>, 1, smem_hb)                    \
-                  : run(k_spectrum<T, NS, false, false>, 1, smem)
+#define SW_SPEC_FORMS(T, NS)                                                  \
+    return f.cluster > 1 ? run(k_spectrum<T, NS, false, true>)                \
+           : f.half      ? run(k_spectrum<T, NS, (NS > 4), false>)            \
+                         : run(k_spectrum<T, NS, false, false>)
     if (lp_kind == 2 || lp_kind == 3) {
-        if (nsig == 16) SW_SPEC_FORMS(__half, 16);
-        if (nsig == 8) SW_SPEC_FORMS(__half, 8);
+        if (f.nsig == 16) SW_SPEC_FORMS(__half, 16);
+        if (f.nsig == 8) SW_SPEC_FORMS(__half, 8);
         SW_SPEC_FORMS(__half, 4);
     }
-    if (nsig == 16) SW_SPEC_FORMS(__nv_bfloat16, 16);
-    if (nsig == 8) SW_SPEC_FORMS(__nv_bfloat16, 8);
+    if (f.nsig == 16) SW_SPEC_FORMS(__nv_bfloat16, 16);
+    if (f.nsig == 8) SW_SPEC_FORMS(__nv_bfloat16, 8);
     SW_SPEC_FORMS(__nv_bfloat16, 4);
 #undef SW_SPEC_FORMS
 }

@@ -1,0 +1,78 @@
+"""The launch rules (sw_forms.h) on the host: tests/c_abi/launch_forms.cpp
+prints their choices for the resident clusters that the runtime reports on a
+GB300 (152 SMs) and for a part with fewer GPCs' worth of them.  No device."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+# SMs, clusters of 1..8 CTAs at one CTA per SM, and at two
+GB300 = [152, 152, 76, 46, 36, 28, 23, 15, 15, 304, 152, 97, 74, 58, 46, 38, 36]
+SMALL = [92, 92, 46, 27, 21, 16, 13, 8, 8, 184, 92, 55, 43, 33, 26, 20, 19]
+OPT_IN = 227 * 1024 - 512
+
+
+@pytest.fixture(scope="module")
+def rules(tmp_path_factory):
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if not cxx:
+        pytest.skip("no C++ compiler")
+    exe = str(tmp_path_factory.mktemp("forms") / "launch_forms")
+    subprocess.run([cxx, "-O1", "-std=c++17", "-I",
+                    os.path.join(ROOT, "paper_2503_13756_gb300", "csrc"),
+                    os.path.join(ROOT, "tests", "c_abi", "launch_forms.cpp"), "-o", exe], check=True)
+
+    def ask(device, queries):
+        r = subprocess.run([exe, *map(str, device)], text=True, capture_output=True, check=True,
+                           input="\n".join("%s %d %d %d %d" % q for q in queries))
+        rows = [tuple(map(int, line.split())) for line in r.stdout.splitlines()]
+        assert len(rows) == len(queries)
+        return rows
+    return ask
+
+
+def _cap(device, per_sm, width):
+    return device[8 * (per_sm - 1) + width]
+
+
+@pytest.mark.parametrize("device", [GB300, SMALL], ids=["gb300", "small"])
+def test_projector_clusters_are_resident_at_once(rules, device):
+    for kind, per_sm in (("slice", 1), ("grid", 2)):
+        count = range(1, 400)
+        widths = [w for w, in rules(device, [(kind, nb, 0, 0, 0) for nb in count])]
+        assert widths[0] == 8 and widths[-1] == 1
+        for nb, w in zip(count, widths):
+            assert w in (1, 2, 4, 8)
+            assert w == 1 or nb <= _cap(device, per_sm, w), (kind, nb, w)
+        assert sorted(widths, reverse=True) == widths
+
+
+def _zeros(n, M):  # the FP16 split's rows of a template
+    return n // 2 * (-(-2 * M // 64) * 64 - 2 * M) * 4
+
+
+@pytest.mark.parametrize("device", [GB300, SMALL], ids=["gb300", "small"])
+def test_spectrum_forms_fit_the_device(rules, device):
+    queries = [("spectrum", nb, n, M, _zeros(n, M))
+               for n in (4, 60, 64, 128, 256, 300, 360, 512, 600, 720, 1024)
+               for M in (1, 33, 64, 96, 100, 128, 160, 192, 224, 256, 512, 1024)
+               for nb in (1, 2, 8, 15, 16, 23, 24, 36, 46, 48, 74, 76, 80, 97, 152, 153, 310, 2000)]
+    seen = set()
+    for (_, nb, n, M, _), (ok, nsig, w, half, smem) in zip(queries, rules(device, queries)):
+        assert ok and nsig in (8, 16) and smem <= OPT_IN
+        assert 1 <= w <= min(8, -(-M // (2 * nsig))) and not (half and w > 1)
+        seen.add(w)
+        if w > 1:
+            sets = -(-nb // _cap(device, 2 if smem <= OPT_IN // 2 else 1, w))
+            assert nb <= device[0] and sets <= 4, (nb, n, M, w)
+    assert seen == set(range(1, 9))
+
+
+def test_one_cluster_too_many_is_counted_as_a_second_set(rules):
+    # of clusters of 8 with one CTA per SM, 15 are resident
+    assert rules(GB300, [("slice", 15, 0, 0, 0), ("slice", 16, 0, 0, 0)]) == [(8,), (4,)]
+    # 48 images of eight batches: 46 clusters of 3 fit (79 us), 76 of 2 (51 us; alone 65 us)
+    assert [r[2] for r in rules(GB300, [("spectrum", 46, 360, 256, 0),
+                                        ("spectrum", 48, 360, 256, 0)])] == [3, 2]
