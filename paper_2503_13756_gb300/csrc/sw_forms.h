@@ -19,14 +19,21 @@ struct DeviceForm {
 };
 
 // CTAs per image (a power of two, at most the portable cluster size 8) of the
-// slice projector with the grid in shared memory, one CTA per SM: the widest
-// cluster with room for all nb images at once.  A cluster too many runs after
-// the others: 16 images in clusters of 8, of which 15 are resident, took twice
-// the time of 15 (L = 64, n = 8: 25 us, 15 us in clusters of 4).
-inline int slice_cluster(int nb, const DeviceForm &d)
+// slice projector with a grid of N x N points in shared memory, one CTA per SM,
+// and nh angles of nj samples: the widest cluster with room for all nb images at
+// once.  A cluster too many runs after the others:
+// 16 images in clusters of 8, of which 15 are resident, took twice the time of
+// 15 (L = 64, n = 8: 25 us, 15 us in clusters of 4).  The barriers and the copies
+// of rows take some us, so an image of little work (the grid's FFTs and the
+// samples, about us of one CTA) stays on its CTA: L = 32, n = 8, 20 images 10 us
+// alone and 12 us in clusters of 4, 46 images 10 and 13 us in clusters of 2; L = 16,
+// n = 360 19 and 12, 20 and 22; L = 64, n = 60 15 and 14, 16 and 17; L = 64, n = 180
+// 27 and 16, 27 and 22.
+inline int slice_cluster(int nb, int N, int nh, int nj, const DeviceForm &d)
 {
+    const double work = 0.00035 * N * N + 0.0032 * nj * nh;
     for (int P = 8; P > 1; P /= 2)
-        if (nb <= d.clusters[0][P]) return P;
+        if (nb <= d.clusters[0][P]) return work >= (P == 2 ? 10.5 : 5.0) ? P : 1;
     return 1;
 }
 

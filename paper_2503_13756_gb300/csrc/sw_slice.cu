@@ -956,7 +956,7 @@ cudaError_t launch_small(SliceArgs a, int nb, cudaStream_t st)
     cudaError_t e = device_form(&dev);
     if (e != cudaSuccess) return e;
     a.pf_ahead = dev->sms;  // resident CTAs: one per SM
-    const int P = slice_cluster(nb, *dev);
+    const int P = slice_cluster(nb, 32 * M, a.nh, 16 * M + 1, *dev);
     const size_t smem = slice_smem_bytes(32 * M);
     return P > 1 ? launch_cluster(k_project_slice<M, true>, nb, P, kSliceThreads, smem, a, st)
                  : launch_cluster(k_project_slice<M, false>, nb, 1, kSliceThreads, smem, a, st);
@@ -969,7 +969,7 @@ cudaError_t launch_up(SliceArgs a, int nb, cudaStream_t st)
     cudaError_t e = device_form(&dev);
     if (e != cudaSuccess) return e;
     a.pf_ahead = dev->sms;
-    const int P = slice_cluster(nb, *dev);
+    const int P = slice_cluster(nb, 32 * MG, a.nh, 32 * MG + 1, *dev);
     const size_t smem = slice_up_smem_bytes(64 * MG);
     return P > 1 ? launch_cluster(k_project_slice_up<MG, true>, nb, P, kSliceThreads, smem, a, st)
                  : launch_cluster(k_project_slice_up<MG, false>, nb, 1, kSliceThreads, smem, a, st);

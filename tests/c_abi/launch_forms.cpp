@@ -18,7 +18,7 @@ int main(int argc, char **argv)
     int a, b, c, e;
     while (scanf("%31s %d %d %d %d", kind, &a, &b, &c, &e) == 5) {
         if (!strcmp(kind, "slice")) {
-            printf("%d\n", swk::slice_cluster(a, d));
+            printf("%d\n", swk::slice_cluster(a, b, c, b / 2 + 1, d));  // b: N, c: nh
         } else if (!strcmp(kind, "grid")) {
             printf("%d\n", swk::slice_grid_cluster(a, d));
         } else if (!strcmp(kind, "spectrum")) {

@@ -41,7 +41,7 @@ def _cap(device, per_sm, width):
 def test_projector_clusters_are_resident_at_once(rules, device):
     for kind, per_sm in (("slice", 1), ("grid", 2)):
         count = range(1, 400)
-        widths = [w for w, in rules(device, [(kind, nb, 0, 0, 0) for nb in count])]
+        widths = [w for w, in rules(device, [(kind, nb, 96, 180, 0) for nb in count])]
         assert widths[0] == 8 and widths[-1] == 1
         for nb, w in zip(count, widths):
             assert w in (1, 2, 4, 8)
@@ -72,7 +72,15 @@ def test_spectrum_forms_fit_the_device(rules, device):
 
 def test_one_cluster_too_many_is_counted_as_a_second_set(rules):
     # of clusters of 8 with one CTA per SM, 15 are resident
-    assert rules(GB300, [("slice", 15, 0, 0, 0), ("slice", 16, 0, 0, 0)]) == [(8,), (4,)]
+    assert rules(GB300, [("slice", 15, 96, 180, 0), ("slice", 16, 96, 180, 0)]) == [(8,), (4,)]
     # 48 images of eight batches: 46 clusters of 3 fit (79 us), 76 of 2 (51 us; alone 65 us)
     assert [r[2] for r in rules(GB300, [("spectrum", 46, 360, 256, 0),
                                         ("spectrum", 48, 360, 256, 0)])] == [3, 2]
+
+
+@pytest.mark.parametrize("N,nh,nb,width", [
+    (64, 4, 2, 1), (64, 4, 20, 1), (64, 4, 46, 1), (64, 30, 36, 1),  # 9..13 us alone
+    (96, 30, 20, 4), (96, 30, 46, 1), (32, 180, 20, 4), (32, 180, 46, 1), (96, 90, 20, 4), (96, 90, 46, 2), (192, 4, 2, 8),
+    (192, 180, 76, 2), (192, 180, 77, 1)])
+def test_images_of_little_work_stay_on_their_cta(rules, N, nh, nb, width):
+    assert rules(GB300, [("slice", nb, N, nh, 0)]) == [(width,)]
