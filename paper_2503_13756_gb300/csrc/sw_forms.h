@@ -112,13 +112,25 @@ inline bool spectrum_form(int nb, int n, int M, int nsig_req, long long zeros, c
     }
     if (f->cluster > 1) return true;
 
-    // Half batches where an SM holds fewer than three CTAs and the images take
-    // more than one wave.
-    const bool half = nsig >= 8 && smem > kSmemOptIn / 3 &&
-                      nb > d.sms * (smem > kSmemOptIn / 2 ? 1 : 2);
-    if (half) {
-        f->half = true;
-        f->smem = smem_of(nsig / 2);
+    // Half batches, where the plain form's buffers leave room for fewer than
+    // three CTAs per SM and the images take more than one wave.  Of the plain
+    // form's time: batches of 16 with one plain CTA per SM (n > 440) 0.55..0.92;
+    // with two, only where the half form takes a wave fewer and wastes none of a
+    // batch or the batches are few (M = 64 0.98 and 0.94, M = 100 0.91, but M =
+    // 128..256 1.02..1.08 at 310 and 420 images, and 1.05..1.21 at 600, which fill
+    // two plain waves).  Batches of 8 (n > 512) halve to rows of 16 bytes per store,
+    // and many images then write parts of sectors (1.24 at 420 images and M = 100,
+    // 1.43..1.84 at 420 to 600 and M = 64): only with one plain CTA per SM and at
+    // most two waves, or few levels.  Levels of one half batch always gain.
+    const int ctas = smem > kSmemOptIn / 2 ? 1 : 2, slots = d.sms * ctas;
+    const int halves = (M + nsig - 1) / nsig;  // half batches
+    if (nsig >= 8 && smem > kSmemOptIn / 3 && nb > slots) {
+        const int waves = (nb + slots - 1) / slots, waves_half = (nb + 3 * d.sms - 1) / (3 * d.sms);
+        const bool odd = halves & 1;
+        f->half = halves == 1 ||
+                  (nsig == 16 ? ctas == 1 || (waves_half < waves && (M <= 64 || odd))
+                              : ctas == 1 && (M <= 40 || (odd && waves <= 2)));
+        if (f->half) f->smem = smem_of(nsig / 2);
     }
     return true;
 }

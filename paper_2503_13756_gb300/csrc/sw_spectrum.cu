@@ -243,19 +243,17 @@ __device__ __forceinline__ void stage_levels(const float *__restrict__ qi, int n
 // frequencies k' = c / NSC + (256 / NSC) i in increasing order, batch after
 // batch; every form keeps that order.
 //  - plain: batches of NSC signals, one thread per class.
-//  - HB, where the plain form's buffers leave room for fewer than three CTAs
-//    per SM (n > 256 at NSC = 16): half batches of NSC / 2 signals, so half of
-//    the buffers and more CTAs on an SM.  Lanes l and l + 16 of a warp take
-//    alternate frequencies of a class and exchange their terms, so both hold
-//    its sum, and a thread keeps two classes, one per half of the batch.
-//    10,001 images at n = 512, M = 256: 5.2 ms plain (one CTA of 8 warps per
-//    SM), 4.9 ms with 512 threads on full batches, 3.9 ms in this form.  Not
-//    for images that the plain form holds all at once: their time is that of
-//    one image's batches in turn (128 images at n = 360, M = 256: 68 us plain,
-//    90 us in this form).
+//  - HB: half batches of NSC / 2 signals, so half of the buffers and more CTAs on
+//    an SM, for many images whose plain buffers leave room for fewer than three.
+//    Lanes l and l + 16 of a warp take alternate frequencies of a class and
+//    exchange their terms, so both hold its sum, and a thread keeps two classes,
+//    one per half of the batch.  10,001 images at n = 512, M = 256: 5.2 ms plain
+//    (one CTA of 8 warps per SM), 4.9 ms with 512 threads on full batches, 3.9 ms
+//    in this form.
 //  - CL: few images; the CTAs of a cluster share an image, CTA r taking the
 //    level batches r, r + S, ...; the terms wait in shared memory, and after
 //    the cluster's barrier CTA 0 adds them in order and finishes the image.
+// Which one a launch takes is spectrum_form's choice (sw_forms.h).
 template <typename T, int NSC, bool HB, bool CL>
 __global__ void __launch_bounds__(kSpecThreads, CL ? 2 : 3)
 k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2 *__restrict__ tw,

@@ -44,3 +44,11 @@ def _check(al, n, M, counts, total, **kw):
     (64, 1024, {})])
 def test_spectrum_clusters_of_every_width(al, n, M, kw):
     _check(al, n, M, (1, 13, 14, 21, 22, 26, 27, 34, 35, 44, 45, 56, 72, 73, 95, 96, 150), 320, **kw)
+
+
+# many images: plain and half batches on each side of the rule's lines
+@pytest.mark.parametrize("n,M,kw", [
+    (360, 100, {}), (360, 64, {"precision": "bf16"}), (320, 9, {}), (512, 129, {}),
+    (720, 64, {}), (900, 101, {"precision": "fp32_simt"}), (1000, 20, {"metric": "rfsw2"})])
+def test_spectra_of_many_images(al, n, M, kw):
+    _check(al, n, M, (150, 153, 303, 309, 455, 470, 599), 640, **kw)

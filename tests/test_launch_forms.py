@@ -84,3 +84,20 @@ def test_one_cluster_too_many_is_counted_as_a_second_set(rules):
     (192, 180, 76, 2), (192, 180, 77, 1)])
 def test_images_of_little_work_stay_on_their_cta(rules, N, nh, nb, width):
     assert rules(GB300, [("slice", nb, N, nh, 0)]) == [(width,)]
+
+
+# (n, M, images): us plain and in half batches, GB300
+HALF = [((512, 256, 160), 164, 147), ((480, 64, 1000), 170, 123), ((500, 100, 310), 250, 184),
+        ((360, 100, 420), 147, 133), ((360, 64, 420), 47, 45), ((900, 100, 160), 295, 266),
+        ((1000, 4, 2000), 944, 575), ((320, 4, 600), 98, 88), ((1000, 33, 1000), 829, 629)]
+PLAIN = [((360, 256, 420), 145, 156), ((320, 192, 600), 121, 147), ((600, 64, 600), 90, 139),
+         ((768, 64, 600), 104, 223), ((720, 128, 420), 154, 274), ((1024, 64, 600), 188, 340),
+         ((900, 64, 420), 133, 178), ((640, 192, 310), 203, 254), ((360, 256, 200), 92, 116)]
+
+
+@pytest.mark.parametrize("size,plain,half", HALF + PLAIN)
+def test_half_batches_where_they_are_faster(rules, size, plain, half):
+    n, M, nb = size
+    ok, _, w, got, smem = rules(GB300, [("spectrum", nb, n, M, _zeros(n, M))])[0]
+    assert ok and w == 1 and smem <= OPT_IN
+    assert got == (half < plain)
