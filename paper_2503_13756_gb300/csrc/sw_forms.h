@@ -58,6 +58,7 @@ struct SpectrumForm {
     int nsig;      // signals per FFT batch
     int cluster;   // CTAs per image
     bool half;     // half batches
+    bool dense;    // four CTAs per SM (plain form)
     size_t smem;   // dynamic shared memory of a CTA
 };
 
@@ -78,7 +79,7 @@ inline bool spectrum_form(int nb, int n, int M, int nsig_req, long long zeros, c
     while (nsig > 4 && smem_of(nsig) > kSmemOptIn) nsig /= 2;
     const size_t smem = smem_of(nsig);
     if (smem > kSmemOptIn) return false;
-    *f = SpectrumForm{nsig, 1, false, smem};
+    *f = SpectrumForm{nsig, 1, false, false, smem};
     const int nbatch = (M + 2 * nsig - 1) / (2 * nsig);
 
     // A cluster per image where it is expected to save a tenth of the time, by
@@ -132,6 +133,12 @@ inline bool spectrum_form(int nb, int n, int M, int nsig_req, long long zeros, c
                               : ctas == 1 && (M <= 40 || (odd && waves <= 2)));
         if (f->half) f->smem = smem_of(nsig / 2);
     }
+
+    // Four CTAs per SM, by 64 registers a thread instead of 80, where shared
+    // memory holds them (n <= 200) and three do not hold all images.  Of the time
+    // at three: n = 8..32 0.69..0.76 at 520 and 600 images, 0.80..0.84 at 1000, n =
+    // 128 0.91 and 0.93, n = 200 0.94 and 0.96; up to 456 images 0.99..1.04.
+    f->dense = !f->half && 4 * (smem + 1536) <= 228 * 1024 && nb > 3 * d.sms;
     return true;
 }
 

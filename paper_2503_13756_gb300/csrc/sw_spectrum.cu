@@ -242,7 +242,8 @@ __device__ __forceinline__ void stage_levels(const float *__restrict__ qi, int n
 // terms: with NSC signals to a batch, signal c mod NSC of each batch at the
 // frequencies k' = c / NSC + (256 / NSC) i in increasing order, batch after
 // batch; every form keeps that order.
-//  - plain: batches of NSC signals, one thread per class.
+//  - plain: batches of NSC signals, one thread per class, three or four CTAs
+//    per SM.
 //  - HB: half batches of NSC / 2 signals, so half of the buffers and more CTAs on
 //    an SM, for many images whose plain buffers leave room for fewer than three.
 //    Lanes l and l + 16 of a warp take alternate frequencies of a class and
@@ -254,8 +255,8 @@ __device__ __forceinline__ void stage_levels(const float *__restrict__ qi, int n
 //    level batches r, r + S, ...; the terms wait in shared memory, and after
 //    the cluster's barrier CTA 0 adds them in order and finishes the image.
 // Which one a launch takes is spectrum_form's choice (sw_forms.h).
-template <typename T, int NSC, bool HB, bool CL>
-__global__ void __launch_bounds__(kSpecThreads, CL ? 2 : 3)
+template <typename T, int NSC, bool HB, bool CL, int CTAS = CL ? 2 : 3>
+__global__ void __launch_bounds__(kSpecThreads, CTAS)
 k_spectrum(const float *__restrict__ q, int n, int M, FftPlan plan, const float2 *__restrict__ tw,
            SpecOut o, float *__restrict__ prof, double *__restrict__ center,
            double *__restrict__ norm32, double *__restrict__ norm16, int parts,
@@ -525,6 +526,7 @@ cudaError_t launch_spectrum(const float *q, int nb, int n, int M, const FftPlan 
 #define SW_SPEC_FORMS(T, NS)                                                  \
     return f.cluster > 1 ? run(k_spectrum<T, NS, false, true>)                \
            : f.half      ? run(k_spectrum<T, NS, (NS > 4), false>)            \
+           : f.dense     ? run(k_spectrum<T, NS, false, false, 4>)            \
                          : run(k_spectrum<T, NS, false, false>)
     if (lp_kind == 2 || lp_kind == 3) {
         if (f.nsig == 16) SW_SPEC_FORMS(__half, 16);

@@ -24,7 +24,7 @@ int main(int argc, char **argv)
         } else if (!strcmp(kind, "spectrum")) {
             swk::SpectrumForm f{};
             const bool ok = swk::spectrum_form(a, b, c, 0, e, d, &f);  // e: zeros per image
-            printf("%d %d %d %d %zu\n", ok, f.nsig, f.cluster, f.half, f.smem);
+            printf("%d %d %d %d %d %zu\n", ok, f.nsig, f.cluster, f.half, f.dense, f.smem);
         } else {
             return 3;
         }

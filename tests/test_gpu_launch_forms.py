@@ -49,6 +49,7 @@ def test_spectrum_clusters_of_every_width(al, n, M, kw):
 # many images: plain and half batches on each side of the rule's lines
 @pytest.mark.parametrize("n,M,kw", [
     (360, 100, {}), (360, 64, {"precision": "bf16"}), (320, 9, {}), (512, 129, {}),
+    (64, 129, {}), (200, 96, {"metric": "rfsw2"}), (8, 256, {"precision": "bf16"}),
     (720, 64, {}), (900, 101, {"precision": "fp32_simt"}), (1000, 20, {"metric": "rfsw2"})])
 def test_spectra_of_many_images(al, n, M, kw):
     _check(al, n, M, (150, 153, 303, 309, 455, 470, 599), 640, **kw)

@@ -60,9 +60,10 @@ def test_spectrum_forms_fit_the_device(rules, device):
                for M in (1, 33, 64, 96, 100, 128, 160, 192, 224, 256, 512, 1024)
                for nb in (1, 2, 8, 15, 16, 23, 24, 36, 46, 48, 74, 76, 80, 97, 152, 153, 310, 2000)]
     seen = set()
-    for (_, nb, n, M, _), (ok, nsig, w, half, smem) in zip(queries, rules(device, queries)):
+    for (_, nb, n, M, _), (ok, nsig, w, half, dense, smem) in zip(queries, rules(device, queries)):
         assert ok and nsig in (8, 16) and smem <= OPT_IN
-        assert 1 <= w <= min(8, -(-M // (2 * nsig))) and not (half and w > 1)
+        assert 1 <= w <= min(8, -(-M // (2 * nsig))) and (w > 1) + half + dense <= 1
+        assert not dense or 4 * (smem + 1024 + 160) <= 228 * 1024  # 1 KB is the system's
         seen.add(w)
         if w > 1:
             sets = -(-nb // _cap(device, 2 if smem <= OPT_IN // 2 else 1, w))
@@ -98,6 +99,16 @@ PLAIN = [((360, 256, 420), 145, 156), ((320, 192, 600), 121, 147), ((600, 64, 60
 @pytest.mark.parametrize("size,plain,half", HALF + PLAIN)
 def test_half_batches_where_they_are_faster(rules, size, plain, half):
     n, M, nb = size
-    ok, _, w, got, smem = rules(GB300, [("spectrum", nb, n, M, _zeros(n, M))])[0]
+    ok, _, w, got, _, smem = rules(GB300, [("spectrum", nb, n, M, _zeros(n, M))])[0]
     assert ok and w == 1 and smem <= OPT_IN
     assert got == (half < plain)
+
+
+# (n, M, images): us at three and at four CTAs per SM, GB300
+@pytest.mark.parametrize("size,three,four", [
+    ((32, 1024, 600), 141, 106), ((8, 1024, 600), 88, 59), ((64, 512, 600), 90, 78),
+    ((128, 33, 600), 63, 59), ((32, 1024, 420), 90, 90), ((128, 33, 420), 49, 49),
+    ((216, 33, 600), 100, 100), ((256, 128, 1000), 96, 100)])
+def test_four_ctas_per_sm_where_they_are_faster(rules, size, three, four):
+    n, M, nb = size
+    assert rules(GB300, [("spectrum", nb, n, M, _zeros(n, M))])[0][4] == (four < three)
