@@ -142,4 +142,13 @@ inline bool spectrum_form(int nb, int n, int M, int nsig_req, long long zeros, c
     return true;
 }
 
+// The ramp filter (k_ramp) of rows of B bins: FFT stages in pairs?  Pairs save
+// passes and barriers but hold twice the registers (64 against 32, four CTAs per
+// SM against eight) and leave most threads of a short row's pass idle.  Time in
+// pairs over single stages, 24 and 1500 images at n = 360: B = 32 1.39 and 1.60, B
+// = 64 1.34 and 1.50, B = 120 1.15 and 1.26; B = 128 1.19 and 1.08, B = 192 1.10
+// and 1.07, B = 256 1.01 and 0.92, B = 384 0.94 and 0.94.  At 600 images, one wave
+// in pairs, 0.95..1.00 at B = 108..192 and 0.89..0.94 above.
+inline bool ramp_pairs(int B) { return B >= 128; }
+
 }  // namespace swk

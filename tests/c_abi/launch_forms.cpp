@@ -25,6 +25,8 @@ int main(int argc, char **argv)
             swk::SpectrumForm f{};
             const bool ok = swk::spectrum_form(a, b, c, 0, e, d, &f);  // e: zeros per image
             printf("%d %d %d %d %d %zu\n", ok, f.nsig, f.cluster, f.half, f.dense, f.smem);
+        } else if (!strcmp(kind, "ramp")) {
+            printf("%d\n", swk::ramp_pairs(a));
         } else {
             return 3;
         }

@@ -7,7 +7,9 @@ here), the same doubles."""
 import numpy as np
 import pytest
 
-from paper_2503_13756_gb300 import swalign
+import oracle
+from paper_2503_13756_gb300 import swalign, synth
+from tests.parity import level_of, rfsw_level_tol
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -53,3 +55,24 @@ def test_spectrum_clusters_of_every_width(al, n, M, kw):
     (720, 64, {}), (900, 101, {"precision": "fp32_simt"}), (1000, 20, {"metric": "rfsw2"})])
 def test_spectra_of_many_images(al, n, M, kw):
     _check(al, n, M, (150, 153, 303, 309, 455, 470, 599), 640, **kw)
+
+
+@pytest.mark.parametrize("B", [120, 128])
+@pytest.mark.parametrize("n", [4, 36])
+def test_ramp_rows_on_each_side_of_the_line(al, B, n):
+    """Quantiles of the ramp-filtered parts against the FP64 oracle's, with FFT
+    stages taken singly (below 128 bins) and in pairs."""
+    L, M = 80, 24
+    p = synth.draw_mixtures(np.random.default_rng(B + n), 3, L, ncomp=(2, 5))
+    imgs = np.ascontiguousarray(synth.render(p, L), dtype=np.float32)
+    par = swalign.make_params(L, n, M, n_bins=B, metric="rfsw2")
+    Q = al.quantiles(al.project(imgs, par), par)[0].cpu().numpy()
+    z = (np.arange(M) + 0.5) / M
+    for i in range(len(imgs)):
+        F, _ = oracle.prepare(imgs[i].astype(np.float64))
+        U = oracle.project(F, n, B)
+        Ut, parts = oracle.ramp_filter(U), oracle.rfsw_parts(U)
+        for part in range(2):
+            for k in range(n):
+                lev = level_of(Q[i, part, k].astype(np.float64), parts[part][k], 2.0 / L)
+                assert np.abs(lev - z).max() <= rfsw_level_tol(Ut[k], parts[part][k]), (i, part, k)

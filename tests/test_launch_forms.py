@@ -112,3 +112,10 @@ def test_half_batches_where_they_are_faster(rules, size, plain, half):
 def test_four_ctas_per_sm_where_they_are_faster(rules, size, three, four):
     n, M, nb = size
     assert rules(GB300, [("spectrum", nb, n, M, _zeros(n, M))])[0][4] == (four < three)
+
+
+# bins: us of 1500 images at n = 360 in pairs of stages and in single stages, GB300
+@pytest.mark.parametrize("B,pairs,single", [
+    (20, 263, 163), (32, 312, 196), (64, 386, 257), (96, 511, 384), (120, 607, 482), (256, 665, 726), (384, 1435, 1530)])
+def test_ramp_stages_in_pairs_where_they_are_faster(rules, B, pairs, single):
+    assert rules(GB300, [("ramp", B, 0, 0, 0)]) == [(pairs < single,)]
