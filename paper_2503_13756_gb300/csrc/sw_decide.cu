@@ -23,6 +23,7 @@
 //    the staging.
 //  - shared-memory form (any n): one CTA per (query, 2*nsig templates), the
 //    mixed-radix Stockham FFT of the library over nsig signals.
+#include "sw_forms.h"
 #include "sw_internal.cuh"
 #include "swalign.h"
 
@@ -762,8 +763,8 @@ k_decide_reg(DecideArgs A, const float2 *__restrict__ tw)
 
 // Best template per query: lowest d2 among usable templates, lowest j on
 // ties.  WQ warps per query (1, or 8: a block): a lane reads every 32 WQ-th
-// result, one after the other, so with many templates the time is that chain
-// (1000 templates: 12 us with a warp, 8 us with a block).
+// result, one after the other, so with many templates the time of a few queries
+// is that chain (1000 templates: 12 us with a warp, 8 us with a block).
 constexpr int kBestThreads = 256;
 template <int WQ>
 __global__ void __launch_bounds__(kBestThreads)
@@ -929,7 +930,10 @@ cudaError_t launch_best_template(const void *all, int Nq, int Nt, void *out, cud
     if (Nq <= 0) return cudaSuccess;
     const auto *res = reinterpret_cast<const sw_result *>(all);
     auto *best = reinterpret_cast<sw_result *>(out);
-    if (Nt > 128)  // more than four results a lane
+    const DeviceForm *dev;
+    const cudaError_t e = device_form(&dev);
+    if (e != cudaSuccess) return e;
+    if (best_by_block(Nq, Nt, *dev))
         return launch_chained(k_best_template<kBestThreads / 32>, dim3(Nq), dim3(kBestThreads), 0, st,
                               1, res, Nq, Nt, best);
     return launch_chained(k_best_template<1>, dim3((Nq * 32 + kBestThreads - 1) / kBestThreads),

@@ -151,4 +151,16 @@ inline bool spectrum_form(int nb, int n, int M, int nsig_req, long long zeros, c
 // in pairs, 0.95..1.00 at B = 108..192 and 0.89..0.94 above.
 inline bool ramp_pairs(int B) { return B >= 128; }
 
+// The best template of Nq queries among Nt (k_best_template): a block per query
+// instead of a warp?  A warp reads its results in chains of Nt / 32, a block in
+// chains of Nt / 256 but with eight warps and a barrier per query, so the block
+// gains while the chip is not filled with blocks.  Block and warp in us: 150 queries
+// of 129 and 1000 templates 4 and 4, 8 and 10; 600 of 129 and 1000 8 and 4, 10
+// and 10; 4000 of 129 and 1000 31 and 10, 51 and 39; 1000 of 2000 21 and 22; 4000
+// of 4000 113 and 131.
+inline bool best_by_block(int Nq, int Nt, const DeviceForm &d)
+{
+    return Nt > 128 && (Nq <= d.sms + Nt / 2 || Nt >= 4000);
+}
+
 }  // namespace swk

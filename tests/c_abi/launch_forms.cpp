@@ -27,6 +27,8 @@ int main(int argc, char **argv)
             printf("%d %d %d %d %d %zu\n", ok, f.nsig, f.cluster, f.half, f.dense, f.smem);
         } else if (!strcmp(kind, "ramp")) {
             printf("%d\n", swk::ramp_pairs(a));
+        } else if (!strcmp(kind, "best")) {
+            printf("%d\n", swk::best_by_block(a, b, d));
         } else {
             return 3;
         }

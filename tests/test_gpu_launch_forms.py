@@ -76,3 +76,23 @@ def test_ramp_rows_on_each_side_of_the_line(al, B, n):
             for k in range(n):
                 lev = level_of(Q[i, part, k].astype(np.float64), parts[part][k], 2.0 / L)
                 assert np.abs(lev - z).max() <= rfsw_level_tol(Ut[k], parts[part][k]), (i, part, k)
+
+
+@pytest.mark.parametrize("nt,counts", [(129, (216, 217)), (300, (302, 303))])
+def test_best_template_on_each_side_of_the_line(al, nt, counts):
+    """A block or a warp per query: the least d2 of the usable results, the
+    lowest index on ties (every third template is a copy of the first)."""
+    g = torch.Generator(device="cuda").manual_seed(nt)
+    p = swalign.make_params(8, 8, 4)
+    t = torch.rand((nt, 8, 8), generator=g, device="cuda")
+    t[::3] = t[0]
+    t[1] = 0.0
+    q = torch.cat([t[:3], torch.rand((counts[-1] - 3, 8, 8), generator=g, device="cuda")])
+    every = swalign.results_to_numpy(al.align_batch(q, t, p)).reshape(-1, nt)
+    j = np.where(every["status"] == 0, every["d2"], np.inf).argmin(1)
+    for count in counts:
+        best = swalign.results_to_numpy(al.align_batch(q[:count].clone(), t, p, mode=1))
+        use = best["status"] == 0
+        assert np.array_equal(use, every["status"][:count].min(1) == 0)
+        assert np.array_equal(best["template_index"][use], j[:count][use])
+        assert np.array_equal(best["d2"][use], every["d2"][np.arange(count), j[:count]][use])

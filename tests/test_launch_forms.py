@@ -119,3 +119,12 @@ def test_four_ctas_per_sm_where_they_are_faster(rules, size, three, four):
     (20, 263, 163), (32, 312, 196), (64, 386, 257), (96, 511, 384), (120, 607, 482), (256, 665, 726), (384, 1435, 1530)])
 def test_ramp_stages_in_pairs_where_they_are_faster(rules, B, pairs, single):
     assert rules(GB300, [("ramp", B, 0, 0, 0)]) == [(pairs < single,)]
+
+
+# (queries, templates): us with a block and with a warp per query, GB300
+@pytest.mark.parametrize("Nq,Nt,block,warp", [
+    (600, 129, 8, 4), (4000, 129, 31, 10), (100, 256, 4, 6), (4000, 256, 31, 12),
+    (150, 500, 6, 8), (1000, 500, 12, 8), (30, 1000, 6, 10), (2000, 1000, 27, 18),
+    (4000, 1000, 51, 39), (600, 4000, 22, 39)])
+def test_best_template_by_block_where_it_is_faster(rules, Nq, Nt, block, warp):
+    assert rules(GB300, [("best", Nq, Nt, 0, 0)]) == [(block < warp,)]
