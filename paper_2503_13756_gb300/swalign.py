@@ -150,11 +150,15 @@ def _ptr(t):
 
 def _stream(stream=None):
     """The handle of the stream, or of the caller's current stream (read
-    without building a Stream object: 0.1 us instead of 3)."""
+    without building a Stream object, 0.1 us instead of 3, where this torch has
+    the private call for it)."""
     import torch
     if stream is not None:
         return stream.cuda_stream
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
 
 
 def _f32(x, device):
