@@ -155,10 +155,10 @@ def _stream(stream=None):
     import torch
     if stream is not None:
         return stream.cuda_stream
-    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-    if raw is None:
+    try:
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    except AttributeError:
         return torch.cuda.current_stream().cuda_stream
-    return raw(torch.cuda.current_device())
 
 
 def _f32(x, device):
