@@ -477,6 +477,17 @@ cudaError_t launch_chained(void (*kern)(K...), dim3 grid, dim3 block, size_t sme
     return cudaGetLastError();
 }
 
+// The quantile kernel's FP32 count of the levels below a node of the CDF, M F /
+// F_B rounded to the nearest integer, is exact unless the quotient lies further
+// than this from that integer (near a boundary between two counts).  Relative
+// error in units of 2^-24: F and F_B without their tails 1 each and the product 1
+// (half an ulp is a unit on a mantissa near 1), the fast quotient's two ulps 4: 7
+// units, 4.2e-7.
+__host__ __device__ __forceinline__ float count_edge(int M)
+{
+    return 0.5f - 4.5e-7f * (float)(M + 1);
+}
+
 // The launch rules' view of the current device (sw_forms.h), asked of the
 // runtime once per device and kept for the process.
 struct DeviceForm;

@@ -158,7 +158,7 @@ __device__ __forceinline__ void load_bins(float (&u)[C], const float *__restrict
 //    number of records apart (no bank conflicts);
 //  - the level counts: M F_j / F_B in FP32 rounded to the nearest count, exact
 //    unless it lands within its rounding error of a boundary between two
-//    counts; a warp in which one does (about one row in a hundred) recounts
+//    counts (count_edge); a warp in which one does (about one row in a hundred) recounts
 //    its row, that node by a double-float comparison with the one level
 //    (by bisection over the levels it took a quarter of the kernel's time);
 //  - two levels at a time in two-wide FP32 operations, and predicated slot
@@ -199,10 +199,7 @@ k_quantiles(const float *__restrict__ proj, int n, int B, int M, float h, int le
     lv.rule = level_rule;
     const float coff = level_rule == 0 ? 0.f : -0.5f;
     const float kstep = level_rule == 0 ? 2.f : 1.f, kofs = level_rule == 0 ? -1.f : 0.f;
-    // distance of the FP32 count from a half-integer below which it is not
-    // trusted: the relative rounding (units of 2^-24) of F's and F_B's tails
-    // (1/2 each), the product (1/2) and the fast quotient (4)
-    const float edge = 0.5f - 4e-7f * (float)(M + 1);
+    const float edge = count_edge(M);
     const float e0 = ((float)c0 - 0.5f * (float)B);
 
     for (int g = 0; g < ngrp; ++g)
