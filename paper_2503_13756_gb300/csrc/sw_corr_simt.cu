@@ -13,6 +13,7 @@
 // of the next stage.
 #include <algorithm>
 
+#include "sw_forms.h"
 #include "sw_internal.cuh"
 
 namespace swk {
@@ -103,7 +104,7 @@ k_corr_simt(const float *__restrict__ X, size_t xf, const float *__restrict__ Y,
 // all padding its time is the latency of its stages (a pair at n = 360, M =
 // 128: 31 us); here a CTA copies the rows of `fb` frequencies to shared memory
 // at once and each thread runs one chain of 2 M dependent FMAs per component
-// (4 us).  Rows are 2 M floats; a frequency's rows take an odd number of
+// (8 us).  Rows are 2 M floats; a frequency's rows take an odd number of
 // floats, so that the threads of adjacent frequencies read distinct banks.
 __global__ void __launch_bounds__(256)
 k_corr_few(const float *__restrict__ X, size_t xf, const float *__restrict__ Y, size_t yf, int Nq,
@@ -142,11 +143,16 @@ cudaError_t launch_corr_simt(const float *X, size_t xf, const float *Y, size_t y
 {
     if (Nq <= 0 || Nt <= 0 || nf <= 0) return cudaSuccess;
     // few pairs: frequencies per CTA so that its rows fit 48 KB and the chip
-    // has a CTA or two per SM (see k_corr_few)
+    // has a CTA or two per SM (see k_corr_few).  Few and tile form in us, at n =
+    // 360, M = 256: 1 x 1 9 and 57, 4 x 4 17 and 57, 8 x 8 26 and 57, 16 x 4 28 and 57, 4
+    // x 16 34 and 57; at n = 256, M = 32 5 to 8 and 8; at n = 60, M = 16 5 to 6 and 6.
+    const DeviceForm *dev;
+    const cudaError_t e = device_form(&dev);
+    if (e != cudaSuccess) return e;
     const size_t per_f = sizeof(float) * ((size_t)(Nq + Nt) * 2 * M + 1);
     if (Nq <= 16 && Nt <= 16 && Nq * Nt <= 64 && per_f <= 48 * 1024) {
         const int fb = (int)std::max<size_t>(
-            1, std::min<size_t>({48 * 1024 / per_f, (size_t)(nf + 151) / 152, (size_t)8}));
+            1, std::min<size_t>({48 * 1024 / per_f, (size_t)((nf + dev->sms - 1) / dev->sms), (size_t)8}));
         return launch_chained(k_corr_few, dim3((nf + fb - 1) / fb), dim3(256), per_f * fb, st, 1, X,
                               xf, Y, yf, Nq, Nt, M, nf, fb, C);
     }

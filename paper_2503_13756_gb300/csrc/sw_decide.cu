@@ -890,7 +890,6 @@ cudaError_t launch_decide(const DecideArgs &args, const FftPlan &plan, const flo
         }
 #undef SW_REG_FORMS
 #undef SW_REG_LAUNCH
-        return cudaGetLastError();
     }
     // shared-memory form: 8 signals (16 pairs) per CTA keeps the shared
     // footprint small enough for several CTAs per SM; 4 at n = 1024.  A
@@ -922,7 +921,6 @@ cudaError_t launch_decide(const DecideArgs &args, const FftPlan &plan, const flo
         else SW_DEC_LAUNCH(4, 2, true);
     }
 #undef SW_DEC_LAUNCH
-    return cudaGetLastError();
 }
 
 cudaError_t launch_best_template(const void *all, int Nq, int Nt, void *out, cudaStream_t st)

@@ -439,8 +439,14 @@ __device__ __forceinline__ float2 *fft_smem(float2 *a, float2 *b, const FftPlan 
 // completion (which also makes its writes visible): 1 to 2 us less at every
 // kernel boundary (a 64 x 64 pair 63 -> 53 us, a request of three images 170 ->
 // 156 us).  Every kernel launched by launch_chained calls chain_wait before it
-// touches anything a previous kernel or call may read or write, and so the
-// order of all of them is kept: a kernel completes only after its predecessor.
+// touches anything that a previous kernel or call on the stream may read or
+// write, and so the order of all of them is kept: a kernel completes only after
+// its predecessor.  Before the wait it may read tables that no kernel writes (a
+// context's angle, twiddle and target tables, uploaded when they were built)
+// and prefetch into L2.  The allocation-free call's tables are written by a
+// kernel, and the kernels it launches read them after the wait.  Launched
+// plainly: k_image_scale, k_msw and k_msw_decide, k_project4<true> (the latter
+// three after a memset) and k_noalloc_tables.
 //
 // No kernel lets its successor in before that (griddepcontrol.
 // launch_dependents): the waiting CTAs then hold registers and shared memory

@@ -436,7 +436,10 @@ cudaError_t launch_project(const float *img, int nb, int L, int srcL, int nh, in
     const bool banded = L > kMaxL4 && band_smem <= 200 * 1024;
     if (n % 4 == 0 && (L <= kMaxL4 || banded)) {
         // canonical angles k = 0..n/8; split over CTAs when the batch is
-        // small.  Default target: ~3 resident CTAs per SM on 152 SMs.
+        // small.  Default target: 456 CTAs, one and a half times the two that an SM
+        // of 152 holds (512 threads of 52 registers).  Targets of 304 and 456 in us at
+        // L = 101, n = 240: 64 images 83 and 84, 200 192 and 185, 338 341 and 297, 450 342
+        // and 370; 304, one wave, 232 and 252 (sw_autotune times both).
         const int kc = n / 8 + 1;
         const int want = want_ctas > 0 ? want_ctas : 456;
         const int nbands = banded ? 2 : 1;

@@ -22,6 +22,7 @@
 
 #include <algorithm>
 
+#include "sw_forms.h"
 #include "sw_internal.cuh"
 
 namespace swk {
@@ -163,8 +164,13 @@ __device__ __forceinline__ void load_bins(float (&u)[C], const float *__restrict
 //    (by bisection over the levels it took a quarter of the kernel's time);
 //  - two levels at a time in two-wide FP32 operations, and predicated slot
 //    stores (a branch each took 7% more instructions).
+// CTAs per SM: four (64 registers) to C = 8, three (80) above.  Three and four in us
+// of 1000 images, n = 360, M = 256: C = 6 165 and 159, 7 170 and 180, 8 182 and 180, 9
+// 209 and 208, 10 198 and 200, 11 240 and 262; of 300 images C = 8 59 and 61, 9 68
+// and 69, 10 65 and 69, 11 77 and 86.
+constexpr int quantile_ctas(int C) { return C >= 9 ? 3 : 4; }
 template <int C, int LV>
-__global__ void __launch_bounds__(kQThreads, C >= 9 ? 3 : 4)
+__global__ void __launch_bounds__(kQThreads, quantile_ctas(C))
 k_quantiles(const float *__restrict__ proj, int n, int B, int M, float h, int level_rule,
             int half, int mirror_out, long long nrow, float *__restrict__ q,
             int32_t *__restrict__ status, int status_shift)
@@ -572,13 +578,12 @@ cudaError_t launch_quantiles(const float *proj, int nb, int n, int B, int M, flo
     // n = 256, M = 128 take 374 us in one set, 353 us in 4 to 7 and 374 us in
     // 16; 128 images at n = 360, M = 256, six rows a warp, 34.7 us in one set
     // and 36.8 us in two).
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const DeviceForm *dev;
+    cudaError_t e = device_form(&dev);
     if (e != cudaSuccess) return e;
     const long long nrow = (long long)nb * nang;
-    const int per_sm = std::max(1, std::min(C >= 9 ? 3 : 4, (int)(220 * 1024 / smem)));
-    const long long set = (long long)sms * per_sm;
+    const int per_sm = std::max(1, std::min(quantile_ctas(C), (int)(220 * 1024 / smem)));
+    const long long set = (long long)dev->sms * per_sm;
     const long long share = nrow / (set * nw);
     const long long sets = std::min<long long>(12, std::max<long long>(1, (share + 8) / 16));
     const int grid = (int)std::min<long long>((nrow + nw - 1) / nw, set * sets);
@@ -613,11 +618,14 @@ cudaError_t launch_center_norm(const float *q, int nb, int n, int M, const doubl
                                double *center, double *norm, cudaStream_t st)
 {
     if (nb <= 0) return cudaSuccess;
-    // CTAs per image: enough for four on each of 152 SMs, eight (the portable
+    // CTAs per image: enough for four on each SM, eight (the portable
     // cluster size) at most, and at least four rows to a warp (below that the
     // reductions cost more than the rows: 151 images at n = 96)
+    const DeviceForm *dev;
+    const cudaError_t e = device_form(&dev);
+    if (e != cudaSuccess) return e;
     int S = 1;
-    while (S < 8 && (long long)nb * S < 4 * 152 && 64 * S <= n) S *= 2;
+    while (S < 8 && (long long)nb * S < 4 * dev->sms && 64 * S <= n) S *= 2;
     return launch_chained(k_center_norm, dim3((unsigned)(nb * S)), dim3(256), 0, st, S, q, n, M, cs64,
                           center, norm);
 }

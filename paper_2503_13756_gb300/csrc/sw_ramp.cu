@@ -123,7 +123,6 @@ cudaError_t launch_ramp(const float *proj, int nb, int nh, int B, const FftPlan 
     else if (nsig == 4) SW_RAMP_LAUNCH(4, true);
     else SW_RAMP_LAUNCH(2, true);
 #undef SW_RAMP_LAUNCH
-    return cudaGetLastError();
 }
 
 }  // namespace swk

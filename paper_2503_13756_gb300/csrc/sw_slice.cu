@@ -161,11 +161,13 @@ __device__ __forceinline__ void cp_async4z(float *dst, const float *src, int src
 }
 
 // Phases A and B for one image into the grid G (shared or global memory),
-// by nw warps; returns the image's bad/mass flags of this thread.  stage
-// (shared memory, two bands of L x 33 floats, or null): with 16 warps and no
-// upsampling the image passes through it in 32-column bands by cp.async,
-// band b + 1 in flight while the warps transform band b (one column pair
-// each); otherwise each lane loads its pixels directly.
+// by nw warps; returns the image's bad/mass flags of this thread.  Unless the
+// image is upsampled, it passes through stage (shared memory): with the grid in
+// global memory in 32-column bands by cp.async (two of L x 33 floats), band b + 1 in
+// flight while the 16 warps transform band b (one column pair each); with the
+// grid in shared memory and one CTA per image in 64-column bands (one of L x 65
+// floats, the idle sample buffer).  Otherwise, and in the clusters of the
+// shared-memory grid, each lane loads its pixels directly.
 //
 // CL: the CTAs of a cluster share the image: each takes every P-th column
 // pair (or band) and kept row, and the cluster's barrier separates the
@@ -777,8 +779,9 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_project_slice(SliceArgs A)
 {
     constexpr int N = 32 * M;
     extern __shared__ __align__(16) float2 sms[];
-    const int nj = N / 2 + 1;
+    constexpr int nj = N / 2 + 1;
     static_assert(__alignof__(sms) >= 16, "the grid takes 16-byte stores");
+    static_assert(2 * N / 3 * 65 <= 2 * kSliceBatch * nj, "Xs stages 64 columns of L <= N / 1.5 rows");
     float2 *G = sms;                                        // [rows][S] grid
     float2 *Xs = G + slice_rows(N) * slice_stride(N);       // [kSliceBatch][nj]
     float2 *tw = Xs + kSliceBatch * nj;                     // [N]
@@ -806,8 +809,8 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_project_slice(SliceArgs A)
     }
 }
 
-// Images of side L/2 upsampled 2 x 2 (128 < L): one CTA per image with the
-// grid of the L/2 image (N = 32 MG = B/2 points, A.L = A.srcL = L/2) in
+// Images of side L/2 upsampled 2 x 2 (128 < L): one CTA, or one cluster (CL), per
+// image with the grid of the L/2 image (N = 32 MG = B/2 points, A.L = A.srcL = L/2) in
 // shared memory, the slice samples j <= N of the L x L image from it in
 // kUpBatch-angle batches (slice_samples<UP>), and rows of B = 2 N bins.
 template <int MG, bool CL>
@@ -817,6 +820,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1) k_project_slice_up(SliceArgs
     constexpr int nj = N + 1;
     extern __shared__ __align__(16) float2 sms[];
     static_assert(__alignof__(sms) >= 16, "the grid takes 16-byte stores");
+    static_assert(2 * N / 3 * 65 <= 2 * kUpBatch * nj, "Xs stages 64 columns of L <= N / 1.5 rows");
     float2 *G = sms;                                        // [rows][S] grid
     float2 *Xs = G + slice_rows(N) * slice_stride(N);       // [kUpBatch][nj]
     float2 *tw = Xs + kUpBatch * nj;                        // [N]

@@ -12,7 +12,8 @@
 // is kept apart, so that the rotation-invariant part of the distance is
 // computed later as a direct difference instead of a cancelling sum.
 //
-// Design (GB300): one CTA per image; levels are taken 2*nsig at a time, two
+// Design (GB300): one CTA per image, or a cluster of them when there are few;
+// levels are taken 2*nsig at a time, two
 // real levels packed into one complex signal, FFT'd by the shared-memory
 // Stockham FFT and unpacked by Hermitian symmetry.  The batches are staged
 // by cp.async into two buffers, so that batch b + 1 is in flight while batch
