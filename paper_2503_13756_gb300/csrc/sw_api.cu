@@ -472,6 +472,9 @@ sw_status get_tables(sw_ctx *c, int n, const Tables **out, int variant = 0)
     SW_CUDA(c, cudaMemcpy(t.cs, cs.data(), sizeof(float2) * n, cudaMemcpyHostToDevice));
     SW_CUDA(c, cudaMemcpy(t.cs64, cs64.data(), sizeof(double2) * n, cudaMemcpyHostToDevice));
     SW_CUDA(c, cudaMemcpy(t.tw, tw.data(), sizeof(float2) * n, cudaMemcpyHostToDevice));
+    // a copy from pageable memory returns once it is staged: on a non-blocking
+    // stream nothing else orders the call's kernels after it
+    SW_CUDA(c, cudaStreamSynchronize(cudaStreamLegacy));
     c->tables.push_back(t);
     *out = &c->tables.back();
     return SW_OK;
@@ -602,6 +605,7 @@ sw_status get_slice_tables(sw_ctx *c, const sw_params *p, const SliceTables **ou
         upload(&t.up_goff, upgoff);
         upload(&t.up_tw, uptw);
     }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);  // (see get_tables)
     if (e != cudaSuccess) {
         cudaGetLastError();
         cudaFree(t.psi_inv);
