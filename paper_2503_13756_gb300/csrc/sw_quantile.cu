@@ -147,7 +147,7 @@ __device__ __forceinline__ void load_bins(float (&u)[C], const float *__restrict
 // that reads its bins twice (B > 384).  LV: adjacent levels per lane of each
 // group of 32 LV levels.
 //
-// Bound by instruction issue (607 warp instructions per row at B = 192, M =
+// Bound by instruction issue (614 warp instructions per row at B = 192, M =
 // 128; 1,174 with a binary search per lane and forward walks).  4352 images
 // at n = 256, B = 192, M = 128: 353 us, 584 us before; 10,001 at n = 512, M =
 // 256: 2.01 ms, 4.32 ms before; 3 at n = 360, B = 384, M = 256: 16 us, 55 us
