@@ -437,7 +437,7 @@ __device__ __forceinline__ float2 *fft_smem(float2 *a, float2 *b, const FftPlan 
 // serialisation, a kernel is prepared while its predecessor runs, its CTAs
 // start as the last of the predecessor's end, and they wait here for its
 // completion (which also makes its writes visible): 1 to 2 us less at every
-// kernel boundary (a 64 x 64 pair 63 -> 53 us, a request of three images 170 ->
+// kernel boundary (a 64 x 64 pair 61 -> 50 us, a request of three images 169 ->
 // 156 us).  Every kernel launched by launch_chained calls chain_wait before it
 // touches anything that a previous kernel or call on the stream may read or
 // write, and so the order of all of them is kept: a kernel completes only after
