@@ -21,14 +21,13 @@ struct DeviceForm {
 // CTAs per image (a power of two, at most the portable cluster size 8) of the
 // slice projector with a grid of N x N points in shared memory, one CTA per SM,
 // and nh angles of nj samples: the widest cluster with room for all nb images at
-// once.  A cluster too many runs after the others:
-// 16 images in clusters of 8, of which 15 are resident, took twice the time of
-// 15 (L = 64, n = 8: 25 us, 15 us in clusters of 4).  The barriers and the copies
-// of rows take some us, so an image of little work (the grid's FFTs and the
-// samples, about us of one CTA) stays on its CTA: L = 32, n = 8, 20 images 10 us
-// alone and 12 us in clusters of 4, 46 images 10 and 13 us in clusters of 2; L = 16,
-// n = 360 19 and 12, 20 and 22; L = 64, n = 60 15 and 14, 16 and 17; L = 64, n = 180
-// 27 and 16, 27 and 22.
+// once.  A cluster too many runs after the others: 16 images in clusters of 8, of
+// which 15 are resident, took 25 us at L = 64, n = 8, and 15 us in clusters of 4.
+// The barriers and the copies of rows take some us, so an image of little work
+// (the grid's FFTs and the samples, about us of one CTA) stays on its CTA.  Us
+// alone and in clusters of 4 for 20 images, and of 2 for 46: L = 32, n = 8 10 and
+// 12, 10 and 13; L = 16, n = 360 19 and 12, 20 and 22; L = 64, n = 60 15 and 14, 16
+// and 17; L = 64, n = 180 27 and 16, 27 and 22.
 inline int slice_cluster(int nb, int N, int nh, int nj, const DeviceForm &d)
 {
     const double work = 0.00035 * N * N + 0.0032 * nj * nh;
@@ -53,6 +52,8 @@ inline int slice_grid_cluster(int nb, const DeviceForm &d)
 // The angle spectra (k_spectrum).
 constexpr int kSpecThreads = 256;
 constexpr size_t kSmemOptIn = 227 * 1024 - 512;  // dynamic shared memory of a CTA, beside the static
+// An SM's 228 KB hold k CTAs of smem bytes (beside each the system's 1 KB and the static).
+inline bool spectrum_fits(int k, size_t smem) { return k * (smem + 1536) <= 228 * 1024; }
 
 struct SpectrumForm {
     int nsig;      // signals per FFT batch
@@ -83,8 +84,8 @@ inline bool spectrum_form(int nb, int n, int M, int nsig_req, long long zeros, c
     const int nbatch = (M + 2 * nsig - 1) / (2 * nsig);
 
     // A cluster per image where it is expected to save a tenth of the time, by
-    // the times of a launch in us on a GB300 (fitted at n = 8..1024, M =
-    // 64..1024; 90% of 11658 measured launches within 10% below and 7% above): 7.5 + b
+    // the times of a launch in us on a GB300 (fitted at n = 8..1024, M = 64..1024;
+    // nine in ten of 11,658 measured launches from 10% below to 7% above): 7.5 + b
     // nbatch + z with a CTA per image, b the time of a batch and z that of the
     // padding; 5 + 5 + 0.86 b ceil(nbatch / w) + 0.29 b nbatch + z / w in
     // clusters of w CTAs (two barriers, the longest CTA's batches, the ordered
@@ -100,7 +101,7 @@ inline bool spectrum_form(int nb, int n, int M, int nsig_req, long long zeros, c
     for (int w = 2; w <= std::min(8, nbatch) && nb <= d.sms; ++w) {
         const int per = (nbatch + w - 1) / w;
         const size_t need = smem + per_batch * per;
-        const int fit = need > kSmemOptIn ? 0 : d.clusters[need <= kSmemOptIn / 2 ? 1 : 0][w];
+        const int fit = need > kSmemOptIn ? 0 : d.clusters[spectrum_fits(2, need) ? 1 : 0][w];
         if (fit == 0) continue;
         const int sets = (nb + fit - 1) / fit;
         const double shared = std::min(nb, fit) * w > d.sms ? 1.16 : 1.0;
@@ -138,7 +139,7 @@ inline bool spectrum_form(int nb, int n, int M, int nsig_req, long long zeros, c
     // memory holds them (n <= 200) and three do not hold all images.  Of the time
     // at three: n = 8..32 0.69..0.76 at 520 and 600 images, 0.80..0.84 at 1000, n =
     // 128 0.91 and 0.93, n = 200 0.94 and 0.96; up to 456 images 0.99..1.04.
-    f->dense = !f->half && 4 * (smem + 1536) <= 228 * 1024 && nb > 3 * d.sms;
+    f->dense = !f->half && spectrum_fits(4, smem) && nb > 3 * d.sms;
     return true;
 }
 

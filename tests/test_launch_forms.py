@@ -66,7 +66,7 @@ def test_spectrum_forms_fit_the_device(rules, device):
         assert not dense or 4 * (smem + 1024 + 160) <= 228 * 1024  # 1 KB is the system's
         seen.add(w)
         if w > 1:
-            sets = -(-nb // _cap(device, 2 if smem <= OPT_IN // 2 else 1, w))
+            sets = -(-nb // _cap(device, 2 if 2 * (smem + 1536) <= 228 * 1024 else 1, w))
             assert nb <= device[0] and sets <= 4, (nb, n, M, w)
     assert seen == set(range(1, 9))
 
